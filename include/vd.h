@@ -120,8 +120,10 @@ int vd_code_supported(int K, int beta, const uint32_t *gens_octal);
  * of Sec. III.  Long int8 / 4-bit streams (at least one task of frame pairs
  * per resident warp) run a persistent kernel whose warps pull tasks and trace
  * one task back while decoding the next forward; shorter ones a kernel with
- * one frame pair per lane group (tune->form overrides).  Both give the same
- * bits.
+ * one frame pair per lane group (tune->form overrides).  Streams of few frames
+ * run, unless tune asks for lanes or a form, a kernel that spreads each frame
+ * pair over a quarter warp (K=7) or a warp (K=9) and keeps its survivors in
+ * shared memory.  All give the same bits.
  *   d_llr:    device pointer to the received LLRs of the whole stream, of
  *             llr_type, in transmitted order (kept positions only when the
  *             code is punctured): n_kept(T) values, T = n_info (+K-1 if

@@ -312,6 +312,34 @@ struct Plan {
 // is faster, from one wave up the persistent one, for K=7 and K=9).
 constexpr int64_t kPersistentWaves = 1;
 
+// Streams of few frames take the wide form (vd_wide.cuh) while its blocks
+// make at most this many waves of what the SMs hold at once (shared memory
+// bounds that).  Both forms' times grow with the frame length and no other
+// form gets faster below one of its own waves, so the line is a number of
+// waves.  Measured (GB300, us per call, wide / otherwise): K=7, f = 256:
+// 10^5 bits 22 / 101, 10^6 23 / 97, 4.2 M (1.9 waves) 56 / 98, 8.4 M (3.9) 103 / 106, 16.8 M
+// 193 / 167; K=9, f = 512: 10^5 bits 44 / 335, 10^6 (1.3) 83 / 335, 4.2 M (5.4)
+// 261 / 346, 8.4 M (10.8) 500 / 360.
+constexpr double kWideWavesK7 = 3.5, kWideWavesK9 = 7.0;
+
+int sm_count() {
+    static std::mutex mu;
+    static std::map<int, int> cache;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = cache.find(dev);
+    if (it != cache.end()) return it->second;
+    int n = 0;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return cache[dev] = n;
+}
+
+bool take_wide(int K, int64_t blocks, size_t smem) {
+    const int64_t per_sm = (int64_t)((228u * 1024u) / (smem + 1024u));   // 228 KB an SM, 1 KB of it reserved per block
+    return (double)blocks <= (K == 7 ? kWideWavesK7 : kWideWavesK9) * (double)(sm_count() * std::max<int64_t>(1, per_sm));
+}
+
 // Resident blocks per SM of the persistent stream kernel, per device and shape.
 int persistent_blocks_per_sm(int K, int lanes, bool r4) {
     static std::mutex mu;
@@ -451,6 +479,28 @@ extern "C" vd_status vd_decode(const vd_code *c, const void *d_llr, int llr_type
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "input pre-pass launch");
         llr = (const int8_t *)buf;
+    }
+
+    if (!f32 && (!tune || (tune->lanes == 0 && tune->form == 0))) {   // the library's choice
+        vd::WideParams wp, wide;
+        wp.llr = llr;
+        wp.n_info = n_info;
+        wp.T = pl.T;
+        wp.f = f;
+        wp.v = v;
+        wp.n_win = pl.n_win;
+        wp.n_pairs = pl.n_pairs;
+        wp.flags = flags;
+        wp.out = d_out;
+        wp.pm_out = d_pm;
+        int64_t blocks = 0;
+        size_t smem = 0;
+        bool full = false;
+        if (vd::wide_plan(c->K, wp, &wide, &blocks, &smem, &full) && take_wide(c->K, blocks, smem)) {
+            const cudaError_t e = vd::launch_wide(c->K, wide, blocks, smem, full, cs);
+            if (e != cudaSuccess) return cuda_fail(e, "decode launch");
+            return VD_OK;
+        }
     }
 
     void *surv = nullptr;

@@ -3,6 +3,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 #include "vd_batch.cuh"
+#include "vd_wide.cuh"
 
 namespace vd {
 
@@ -38,6 +39,15 @@ cudaError_t batch_occupancy_k9(int lanes, bool radix4, int *blocks_per_sm);
 cudaError_t launch_stream_persistent(int K, int lanes, bool radix4, const StreamParams &p, int64_t blocks,
                                      cudaStream_t st);
 cudaError_t stream_persistent_occupancy(int K, int lanes, bool radix4, int *blocks_per_sm);
+
+// Wide form (vd_wide.cuh), for streams of few frames: wide_plan fills the
+// padded length, the records kept and the pairs per warp, and says how many
+// blocks of one warp and how much shared memory each takes; false if a
+// frame pair's survivors do not fit.
+constexpr size_t kWideSmemMax = 226u * 1024u;
+bool wide_plan(int K, const WideParams &in, WideParams *out, int64_t *blocks, size_t *smem, bool *full);
+cudaError_t launch_wide(int K, const WideParams &p, int64_t blocks, size_t smem, bool full, cudaStream_t st);
+
 cudaError_t launch_stream_f32_k7(int lanes, const StreamParams &p, int64_t blocks, cudaStream_t st);
 cudaError_t launch_stream_f32_k9(int lanes, const StreamParams &p, int64_t blocks, cudaStream_t st);
 bool geom_f32_k7(int lanes, KernelGeom *g);
