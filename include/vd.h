@@ -123,7 +123,9 @@ int vd_code_supported(int K, int beta, const uint32_t *gens_octal);
  * one frame pair per lane group (tune->form overrides).  Streams of few frames
  * run, unless tune asks for lanes or a form, a kernel that spreads each frame
  * pair over a quarter warp (K=7) or a warp (K=9) and keeps its survivors in
- * shared memory.  All give the same bits.
+ * shared memory; few long frames are decoded in overlapping segments at once,
+ * which run again until their metrics agree with those of the frame decoded in
+ * one piece.  All give the same bits.
  *   d_llr:    device pointer to the received LLRs of the whole stream, of
  *             llr_type, in transmitted order (kept positions only when the
  *             code is punctured): n_kept(T) values, T = n_info (+K-1 if

@@ -496,6 +496,13 @@ extern "C" vd_status vd_decode(const vd_code *c, const void *d_llr, int llr_type
         int64_t blocks = 0;
         size_t smem = 0;
         bool full = false;
+        vd::SplitParams sp;
+        int ranks = 0;
+        if (vd::split_plan(c->K, wp, sm_count(), &sp, &ranks, &smem)) {
+            const cudaError_t e = vd::launch_split(c->K, sp, ranks, smem, cs);
+            if (e != cudaSuccess) return cuda_fail(e, "decode launch");
+            return VD_OK;
+        }
         if (vd::wide_plan(c->K, wp, &wide, &blocks, &smem, &full) && take_wide(c->K, blocks, smem)) {
             const cudaError_t e = vd::launch_wide(c->K, wide, blocks, smem, full, cs);
             if (e != cudaSuccess) return cuda_fail(e, "decode launch");

@@ -48,6 +48,14 @@ constexpr size_t kWideSmemMax = 226u * 1024u;
 bool wide_plan(int K, const WideParams &in, WideParams *out, int64_t *blocks, size_t *smem, bool *full);
 cudaError_t launch_wide(int K, const WideParams &p, int64_t blocks, size_t smem, bool full, cudaStream_t st);
 
+// Split form (vd_wide.cuh): one frame per cluster of `ranks` blocks; false
+// if frames are too many, too short to gain, or too long for a cluster's shared memory.
+// kSplitWarmup: chunks of K-1 stages (96 stages for K=7, 128 for K=9, 14 to 16 constraint lengths): at
+// 2 dB and above hardly a segment runs twice.  kSplitGain: what the checks and barriers cost, in chunks.
+constexpr int kSplitWarmup = 16, kSplitGain = 8;
+bool split_plan(int K, const WideParams &in, int n_sm, SplitParams *out, int *ranks, size_t *smem);
+cudaError_t launch_split(int K, const SplitParams &p, int ranks, size_t smem, cudaStream_t st);
+
 cudaError_t launch_stream_f32_k7(int lanes, const StreamParams &p, int64_t blocks, cudaStream_t st);
 cudaError_t launch_stream_f32_k9(int lanes, const StreamParams &p, int64_t blocks, cudaStream_t st);
 bool geom_f32_k7(int lanes, KernelGeom *g);

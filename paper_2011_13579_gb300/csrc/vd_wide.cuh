@@ -52,6 +52,8 @@
 // chunk's normalisation leaves that frame alone, and its metrics stay
 // within HT + 2 (2 U - 1) B.
 #pragma once
+#include <cooperative_groups.h>
+
 #include "vd_stream.cuh"
 
 namespace vd {
@@ -166,6 +168,9 @@ struct WideForward {
     // stg: this pair's staged words; rec: this lane's words of record rec0
     // (rows of PPW pairs), rec0 the first of a chunk; reset: stage at which frame h
     // starts from the reset state (-1: none).
+    // MODE: keep the records from rec0 on, none of them, or all of them.
+    enum Mode { FROM_REC0, NONE, ALL };
+    template <Mode MODE = FROM_REC0>
     __device__ __forceinline__ static void run(uint32_t (&P)[NR], const uint32_t *stg, int nchunks, uint32_t *rec,
                                                int rec0, int reset0, int reset1, int lane) {
         const uint32_t one = threadIdx.y + 1u;   // 1, unknown to the compiler: keeps multiply-adds on the FMA pipe
@@ -338,15 +343,62 @@ struct WideForward {
         const int ra = (int)(__reduce_min_sync(0xFFFFFFFFu, rlo < 0 ? 0x7FFFFFFFu : (unsigned)rlo) / U);
         const int rz = __reduce_max_sync(0xFFFFFFFFu, rhi) / U;
         for (int c = 0; c < nchunks; ++c) {
+            const bool store = MODE == ALL || (MODE == FROM_REC0 && c >= c0);
             if (c >= ra && c <= rz) {
-                if (c >= c0) chunk(std::true_type{}, std::true_type{}, c);
+                if (store) chunk(std::true_type{}, std::true_type{}, c);
                 else chunk(std::true_type{}, std::false_type{}, c);
-            } else if (c >= c0) {
+            } else if (store) {
                 chunk(std::false_type{}, std::true_type{}, c);
             } else {
                 chunk(std::false_type{}, std::false_type{}, c);
             }
         }
+    }
+
+    // The best state of frame h over the group's L lanes (the lowest index
+    // among equals; states with a bit of `unreach` left out) and the smallest metric.
+    __device__ __forceinline__ static uint32_t best_state(const uint32_t (&P)[NR], int h, int lane, uint32_t unreach,
+                                                          uint32_t &mn) {
+        uint32_t best = 0;
+        mn = 0xFFFFu;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const uint32_t m = h ? (P[r] >> 16) : (P[r] & 0xFFFFu);
+            const uint32_t Rg = ((uint32_t)lane << LR) | (uint32_t)r;
+            const uint32_t key = (Rg & unreach) ? 0u : ((m << 16) | (0xFFFFu - Rg));
+            best = best > key ? best : key;
+            mn = mn < m ? mn : m;
+        }
+#pragma unroll
+        for (int m = 1; m < L; m <<= 1) {
+            const uint32_t x = __shfl_xor_sync(0xFFFFFFFFu, best, m);
+            const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, mn, m);
+            best = best > x ? best : x;
+            mn = mn < y ? mn : y;
+        }
+        return 0xFFFFu - (best & 0xFFFFu);
+    }
+
+    // Traceback over one group of K-1 stages of frame h; rp: the pair's last record of the group.
+    __device__ __forceinline__ static void back(uint32_t &Rc, const uint32_t *&rp, int h) {
+        static_for<NB / ES>([&](auto jc) {
+            constexpr int j = decltype(jc)::value;
+            constexpr int ph0 = NB - ES * (j + 1);   // phase of the record's first stage
+            constexpr uint32_t m = ((1u << ES) - 1u) << ph0;
+            const uint32_t word = rp[Rc / RPW];
+            rp -= PPW * Cfg::ROW;
+            const uint32_t sh = (uint32_t)FW * (Rc & (uint32_t)(RPW - 1)) + 16u * (uint32_t)h;
+            Rc = (Rc & ~m) | (__funnelshift_r(word, word, sh - (uint32_t)ph0) & m);
+        });
+    }
+
+    // Subtracts each frame's smallest metric from all its metrics.
+    __device__ __forceinline__ static void canonical(uint32_t (&P)[NR]) {
+        uint32_t mn = min_tree<NR>(P);
+#pragma unroll
+        for (int m = 1; m < L; m <<= 1) mn = min_u16x2(mn, __shfl_xor_sync(0xFFFFFFFFu, mn, m));
+#pragma unroll
+        for (int r = 0; r < NR; ++r) P[r] -= mn;   // no half is below its minimum: no borrow
     }
 };
 
@@ -356,7 +408,7 @@ __global__ void __launch_bounds__(32, 8) wide_kernel(const WideParams p) {
     using Cfg = WideCfg<K, BETA, GENS, L>;
     using Fw = WideForward<K, BETA, GENS, L, PPW>;
     constexpr int NB = Cfg::NB, NS = Cfg::NS, NR = Cfg::NR, LR = Cfg::LR, ES = Cfg::ES, SC = Cfg::SC;
-    constexpr int LW = Cfg::LW, ROW = Cfg::ROW, FW = Cfg::FW, RPW = Cfg::RPW;
+    constexpr int LW = Cfg::LW, ROW = Cfg::ROW;
     extern __shared__ __align__(16) uint32_t vd_wide_smem[];
     const int wlane = (int)threadIdx.x;
     const int group = wlane / L, lane = wlane % L;
@@ -404,23 +456,9 @@ __global__ void __launch_bounds__(32, 8) wide_kernel(const WideParams p) {
     for (int h = 0; h < 2; ++h) {
         // states a reset frame of fewer than K-1 stages cannot reach are left out
         const uint32_t unreach = (known[h] && W[h] < NB) ? ((1u << (NB - W[h])) - 1u) : 0u;
-        uint32_t best = 0, mn = 0xFFFFu;
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            const uint32_t m = h ? (P[r] >> 16) : (P[r] & 0xFFFFu);
-            const uint32_t Rg = ((uint32_t)lane << LR) | (uint32_t)r;
-            const uint32_t key = (Rg & unreach) ? 0u : ((m << 16) | (0xFFFFu - Rg));
-            best = best > key ? best : key;
-            mn = mn < m ? mn : m;
-        }
-#pragma unroll
-        for (int m = 1; m < L; m <<= 1) {
-            const uint32_t x = __shfl_xor_sync(0xFFFFFFFFu, best, m);
-            const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, mn, m);
-            best = best > x ? best : x;
-            mn = mn < y ? mn : y;
-        }
-        R[h] = term[h] ? 0u : (0xFFFFu - (best & 0xFFFFu));
+        uint32_t mn;
+        const uint32_t best = Fw::best_state(P, h, lane, unreach, mn);
+        R[h] = term[h] ? 0u : best;
         if (p.pm_out && valid[h] && active) {
             int32_t *dst = p.pm_out + (2 * q + h) * NS + ((int64_t)lane << LR);
 #pragma unroll
@@ -442,15 +480,7 @@ __global__ void __launch_bounds__(32, 8) wide_kernel(const WideParams p) {
     const uint32_t *rp = recs + (wpad / ES - 1 - p.rec0) * row;   // the last record
     for (int g = wpad / NB - 1; g >= g0; --g) {
         if ((PPW > 1 || group == 0) && lane < 2) grp[2 * g + h] = (uint8_t)Rc;
-        static_for<NB / ES>([&](auto jc) {
-            constexpr int j = decltype(jc)::value;
-            constexpr int ph0 = NB - ES * (j + 1);   // phase of the record's first stage
-            constexpr uint32_t m = ((1u << ES) - 1u) << ph0;
-            const uint32_t word = rp[Rc / RPW];
-            rp -= row;
-            const uint32_t sh = (uint32_t)FW * (Rc & (uint32_t)(RPW - 1)) + 16u * (uint32_t)h;
-            Rc = (Rc & ~m) | (__funnelshift_r(word, word, sh - (uint32_t)ph0) & m);
-        });
+        Fw::back(Rc, rp, h);
     }
     __syncwarp();
 
@@ -474,6 +504,217 @@ __global__ void __launch_bounds__(32, 8) wide_kernel(const WideParams p) {
             }
         }
     }
+}
+
+// ------------------------------------------------------------- split frames
+//
+// A frame is a serial chain of W stages; where there are few frames and each is
+// long (a packet decoded full length) that chain is all the time there is.
+// Here a cluster of blocks decodes one frame in segments, all at once, and the
+// result is exact:
+//   * a segment of S chunks starts M chunks early from all-equal metrics.
+//     After the warm-up its metrics differ from the true ones by a constant if
+//     every survivor of the warm-up has one ancestor, which is nearly always so;
+//   * a segment's metrics at its start (less their minimum) are compared
+//     with the end of the segment before.  Equal metrics give equal decisions,
+//     so when all agree, every segment is exact, from the first one (which
+//     starts where the frame does) on.  Segments that disagree run again from
+//     the metrics at the end of the segment before, until none disagrees: at
+//     most as many rounds as segments, since each round settles one more;
+//   * each segment is traced back from its best end state at first; then the
+//     segments whose successor's traceback arrives in another state are traced again from
+//     that state, as far as the two paths differ, until none changes.
+// Segments go through the registers in pairs, as frames do in wide_kernel.
+//
+// What bounds it: the warm-up and the segment, (16 + S) (K-1) stages of 80
+// (K=7) or 100 (K=9) cycles, and some five barriers of the cluster.  Four warps a block, one
+// per scheduler (a second one on a scheduler costs 28 cycles a stage); clusters of 1 to 8
+// blocks, as wide as keeps S at half the warm-up.  Measured (us per vd_decode
+// call, this form / wide / one lane per pair): K=7 full length, terminated, 3 dB, 4,096
+// bits 14.7 / 209 / 1172, 30,000 bits 18.7 / - / 8452; K=9, 4,096 bits 20.8 / - /
+// 2148; at 0 dB, where some segments run twice, 28.9 and 33.0.
+struct SplitParams {
+    const int8_t *llr;
+    int64_t n_info, T, f, v;
+    int64_t n_win;
+    uint32_t flags;
+    int32_t S, M;           // chunks of a segment, and of its warm-up
+    uint32_t *out;
+    int32_t *pm_out;
+};
+
+// Words of shared memory of a block of `warps` warps.
+template <int K, int BETA, uint64_t GENS, int L>
+struct SplitSmem {
+    using Cfg = WideCfg<K, BETA, GENS, L>;
+    static constexpr int PPW = 32 / L;
+    int stg, rec, ve, gl, total;   // words per pair / per warp / per pair / in all / in all
+    __host__ __device__ constexpr SplitSmem(int warps, int S, int M)
+        : stg((S + M) * Cfg::U * Cfg::LW), rec(S * (Cfg::U / Cfg::ES) * PPW * Cfg::ROW), ve(Cfg::NS),
+          gl((warps * PPW * 2 * S + 3) / 4),
+          total(warps * (PPW * (stg + ve) + rec) + gl + (warps * PPW * 2 + 3) / 4 + 4) {}
+};
+
+template <int K, int BETA, uint64_t GENS, int L, int MAXT>
+__global__ void __launch_bounds__(MAXT) split_kernel(const SplitParams p) {
+    constexpr int PPW = 32 / L;
+    using Cfg = WideCfg<K, BETA, GENS, L>;
+    using Fw = WideForward<K, BETA, GENS, L, PPW>;
+    constexpr int NB = Cfg::NB, NS = Cfg::NS, NR = Cfg::NR, LR = Cfg::LR, ES = Cfg::ES, SC = Cfg::SC, U = Cfg::U;
+    constexpr int ROW = Cfg::ROW;
+    extern __shared__ __align__(16) uint32_t vd_wide_smem[];
+    auto cluster = cooperative_groups::this_cluster();
+    const int rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
+    const int warps = (int)blockDim.x / 32, warp = (int)threadIdx.x / 32, wlane = (int)threadIdx.x % 32;
+    const int group = wlane / L, lane = wlane % L;
+    const SplitSmem<K, BETA, GENS, L> sm(warps, p.S, p.M);
+    const int pairs = warps * PPW, pair = warp * PPW + group;   // of this block
+    const int gp = rank * pairs + pair;                         // the frame's pair: segments 2 gp, 2 gp + 1
+    const int nseg = 2 * ranks * pairs;
+    uint32_t *stg = vd_wide_smem + pair * sm.stg;
+    uint32_t *recs = vd_wide_smem + pairs * sm.stg + warp * sm.rec + group * ROW;
+    uint32_t *ve = vd_wide_smem + pairs * sm.stg + warps * sm.rec;   // metrics at the segments' ends, by state
+    uint8_t *gl = reinterpret_cast<uint8_t *>(ve + pairs * NS);      // register index at the top of every chunk
+    uint8_t *xs = gl + 4 * sm.gl;                                    // state each segment's traceback arrives in
+    uint32_t *flag = ve + pairs * NS + sm.gl + (pairs * 2 + 3) / 4;
+    auto sync = [&] {
+        if (ranks == 1) __syncthreads();
+        else cluster.sync();
+    };
+    // whether any thread of the cluster says yes; a barrier for all of them
+    int round = 0;
+    auto any_of = [&](bool yes) {
+        const int mine = __syncthreads_or(yes);
+        if (ranks == 1) return mine != 0;
+        uint32_t *f = flag + (round++ & 1);
+        if (threadIdx.x == 0) *f = (uint32_t)mine;
+        cluster.sync();
+        uint32_t all = 0;
+        for (int k = 0; k < ranks; ++k) all |= *cluster.map_shared_rank(f, k);
+        return all != 0;
+    };
+
+    const FrameTask ft = frame_task(p.llr, p.out, nullptr, (int64_t)(blockIdx.x / ranks), p.n_win, p.n_info, p.T, p.f,
+                                    p.v, p.flags);
+    const int W = (int)(ft.b - ft.a);
+    const int wpad = (p.S + p.M) * U, seg = p.S * U;
+    int w[2], reset[2];
+    const int8_t *base[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        // segment i ends (nseg - 1 - i) segments before the frame's end; its window begins
+        // S + M chunks earlier or with the frame
+        const int y = W - (nseg - 1 - (2 * gp + h)) * seg;
+        const int x = y > wpad ? y - wpad : 0;
+        w[h] = y > 0 ? y - x : 0;
+        base[h] = ft.llr + (ft.a + x) * BETA;
+        reset[h] = (ft.known && x == 0 && y > 0) ? wpad - w[h] : -1;
+    }
+    wide_stage_pair<BETA, Cfg::LW, L>(base[0], base[1], w[0], w[1], wpad, stg, lane);
+    __syncwarp();
+
+    // ---- forward: warm-up, then the segment, until its start is the end of the one before
+    uint32_t P[NR], V[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) P[r] = Fw::SEED;
+    Fw::template run<Fw::NONE>(P, stg, p.M, nullptr, 0, reset[0], reset[1], lane);
+    Fw::canonical(P);
+    const int first = p.M * U;
+    const int rs0 = reset[0] >= first ? reset[0] - first : -1, rs1 = reset[1] >= first ? reset[1] - first : -1;
+    bool run = true;
+    while (true) {
+        if (run) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) V[r] = P[r];
+            Fw::template run<Fw::ALL>(P, stg + first * Cfg::LW, p.S, recs + lane * Cfg::NWE, 0, rs0, rs1, lane);
+            Fw::canonical(P);
+#pragma unroll
+            for (int r = 0; r < NR; ++r) ve[pair * NS + ((lane << LR) | r)] = P[r];
+        }
+        sync();
+        const uint32_t *own = ve + pair * NS;
+        const uint32_t *prev = pair > 0 ? own - NS
+                               : rank > 0 ? cluster.map_shared_rank(ve, rank - 1) + (pairs - 1) * NS : nullptr;
+        uint32_t N[NR];
+        bool bad = false;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const int st = (lane << LR) | r;
+            N[r] = (prev ? prev[st] >> 16 : V[r] & 0xFFFFu) | (own[st] << 16);
+            bad |= N[r] != V[r];
+        }
+        run = __any_sync(0xFFFFFFFFu, bad);
+        if (!any_of(run)) break;
+        if (run) {
+#pragma unroll
+            for (int r = 0; r < NR; ++r) P[r] = N[r];
+        }
+    }
+
+    // ---- traceback: lanes 0 and 1 of a group take its two segments
+    const int h = lane & 1;
+    const int si = 2 * gp + h;
+    uint32_t R0 = 0;
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+        uint32_t mn;
+        const uint32_t unreach = (ft.known && W < NB) ? ((1u << (NB - W)) - 1u) : 0u;
+        const uint32_t best = Fw::best_state(P, hh, lane, 2 * gp + hh == nseg - 1 ? unreach : 0u, mn);
+        if (h == hh) R0 = (ft.term && 2 * gp + hh == nseg - 1) ? 0u : best;
+        if (p.pm_out && 2 * gp + hh == nseg - 1) {   // canonical final metrics
+            int32_t *dst = p.pm_out + (int64_t)(blockIdx.x / ranks) * NS + (lane << LR);
+#pragma unroll
+            for (int r = 0; r < NR; ++r) dst[r] = (int32_t)((hh ? (P[r] >> 16) : (P[r] & 0xFFFFu)) - mn) / SC;
+        }
+    }
+    const bool tracer = lane < 2;
+    const uint32_t *last = recs + (p.S * (U / ES) - 1) * (PPW * ROW);
+    uint8_t *mygl = gl + (2 * pair + h) * p.S;
+    if (tracer) {
+        uint32_t Rc = R0;
+        const uint32_t *rp = last;
+        for (int g = p.S - 1; g >= 0; --g) {
+            mygl[g] = (uint8_t)Rc;
+            Fw::back(Rc, rp, h);
+        }
+        xs[2 * pair + h] = (uint8_t)Rc;
+    }
+    while (true) {
+        sync();
+        uint32_t Rc = R0;
+        if (tracer && si < nseg - 1)
+            Rc = 2 * pair + h + 1 < 2 * pairs ? xs[2 * pair + h + 1] : *cluster.map_shared_rank(xs, rank + 1);
+        const bool change = tracer && Rc != R0;
+        if (!any_of(change)) break;
+        if (change) {
+            R0 = Rc;
+            const uint32_t *rp = last;
+            int g = p.S - 1;
+            for (; g >= 0 && mygl[g] != (uint8_t)Rc; --g) {   // from there on the path is the old one
+                mygl[g] = (uint8_t)Rc;
+                Fw::back(Rc, rp, h);
+            }
+            if (g < 0) xs[2 * pair + h] = (uint8_t)Rc;
+        }
+    }
+
+    // ---- decoded words, in turn over the cluster's threads
+    const int per = 2 * pairs * p.S;                   // chunks per block
+    const int pad = nseg * seg - W;                    // stages before the frame's first one
+    const int o = (int)(ft.o - ft.a) + pad, nbits = (int)(ft.e - ft.o);
+    uint32_t *dst = ft.out + (ft.o >> 5);
+    for (int wd = rank * (int)blockDim.x + (int)threadIdx.x; 32 * wd < nbits; wd += ranks * (int)blockDim.x) {
+        const int t = o + 32 * wd, g = t / NB;
+        uint64_t acc = 0;
+        constexpr int NG = (31 + NB - 1) / NB + 1;   // chunks that 32 stages can touch
+#pragma unroll
+        for (int i = 0; i < NG; ++i)
+            if (g + i < ranks * per) acc |= (uint64_t)cluster.map_shared_rank(gl, (g + i) / per)[(g + i) % per] << (NB * i);
+        acc >>= t - g * NB;
+        const int left = nbits - 32 * wd;
+        dst[wd] = (uint32_t)acc & (left >= 32 ? 0xFFFFFFFFu : ((1u << left) - 1u));
+    }
+    if (ranks > 1) cluster.sync();   // no block leaves while another may read its shared memory
 }
 
 }  // namespace vd

@@ -1,5 +1,5 @@
-"""The wide form of vd_decode (few frames, survivors in shared memory) against
-the CPU oracle: decoded bits and canonical final metrics, element by element.
+"""The forms of vd_decode for few frames (a pair over many lanes with its
+survivors in shared memory; long frames in segments) against the CPU oracle: decoded bits and canonical final metrics, element by element.
 
 Sizes sit at the form's edges: streams shorter than the K-1 memory, one pair,
 a pair with one frame, a warp's four pairs (K=7) and one more, frames long
@@ -22,6 +22,10 @@ from paper_2011_13579_gb300 import synth  # noqa: E402
 GENS = {7: synth.K7_GENS, 9: synth.K9_GENS}
 SHAPES = ([(1, 32, 8), (31, 32, 0), (33, 64, 6), (70, 64, 100), (256, 256, 42), (513, 256, 42), (2048, 256, 42), (2049, 256, 42),
            (2999, 3000, 8), (9001, 128, 30)] + [(200 + i, 4096, 8) for i in range(8)] + [(300, 64, v) for v in range(8, 16)])
+# frames decoded in segments: one block's worth, a chunk more than a whole number of segments, clusters of 2 to 8 blocks,
+# several long frames, frames too long for one block's shared memory
+LONG = {7: [(400, 400, 6), (1151, 1151, 6), (4096, 4096, 6), (4601, 4601, 0), (20011, 20011, 6), (9000, 2048, 42), (3000, 640, 700)],
+        9: [(520, 520, 8), (1031, 1031, 8), (4096, 4096, 8), (9001, 9001, 8), (6000, 2048, 64)]}
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -38,6 +42,8 @@ def values(K, n, T, kind, rng):
         return synth.make_stream(rng, K, GENS[K], n, 1.0, T > n).s8()
     if kind == "zeros":
         return np.zeros(beta * T, np.int8)
+    if kind == "faint":      # no codeword and hardly any information: survivors take long to meet, segments run again
+        return rng.integers(-1, 2, beta * T).astype(np.int8) * (rng.random(beta * T) < 0.15)
     if kind == "saturated":
         return (127 * (1 - 2 * rng.integers(0, 2, beta * T))).astype(np.int8)
     q = rng.integers(-127, 128, beta * T).astype(np.int8)
@@ -51,7 +57,19 @@ def values(K, n, T, kind, rng):
 def test_wide_matches_oracle(K, term, unknown, kind):
     rng = np.random.Generator(np.random.PCG64(700 + K + 2 * term + unknown))
     code, oc, beta = vd.Code(K, GENS[K]), oracle.Code(K, GENS[K]), len(GENS[K])
-    for i, (n, f, v) in enumerate(SHAPES):
+    check(K, code, oc, beta, SHAPES, term, unknown, kind, rng)
+
+
+@pytest.mark.parametrize("kind", ["noisy", "zeros", "erasures", "faint"])
+@pytest.mark.parametrize("term,unknown", [(True, False), (False, True)])
+@pytest.mark.parametrize("K", [7, 9])
+def test_segmented_frames_match_oracle(K, term, unknown, kind):
+    rng = np.random.Generator(np.random.PCG64(900 + K + 2 * term + unknown))
+    check(K, vd.Code(K, GENS[K]), oracle.Code(K, GENS[K]), len(GENS[K]), LONG[K], term, unknown, kind, rng)
+
+
+def check(K, code, oc, beta, shapes, term, unknown, kind, rng):
+    for i, (n, f, v) in enumerate(shapes):
         T = n + (K - 1 if term else 0)
         q = values(K, n, T, kind, rng)
         buf = torch.zeros(q.size + 16, dtype=torch.uint8, device="cuda")
