@@ -11,6 +11,14 @@
 // The noise is the k-th standard normal of the stream: Philox4x64-10 (Salmon
 // et al., SC 2011) with key (seed, stream_id) on counter block k / 4, turned
 // into four normals by the Box-Muller transform in double precision.
+//
+// What bounds it: the 64-bit integer products of Philox.  In double precision
+// alone the transform bound it instead (the fp64 units give two lanes per clock and SM): 732 us for
+// 8.4 M int8 values, on GB300.  The transform is therefore taken in single precision with an
+// error bound, which settles the quantised value unless a rounding border
+// lies within the bound; a thread with such a value (2 in 10^4 for int8, 1 in 100 for half
+// precision) takes its eight values from the double-precision transform instead.  The bytes are those of
+// the double-precision transform.  Measured: 8.4 M int8 values (2^22 bits, K=7) 732 -> 76 us.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -29,16 +37,29 @@ struct TxParams {
     uint32_t gens[4];
     uint8_t pos_phase[32], pos_b[32];   // r-th kept position of a period: (phase, output)
     double sigma, inv_var2;             // sigma and 2 / sigma^2
+    float sigma_f, inv_var2_f;
+    uint64_t kpp_magic;                 // 2^64 / kept_per_period, rounded up: k / kept_per_period = high word of k kpp_magic
+    int aligned;                        // out on a 16-byte boundary
     uint64_t seed, stream_id;
-    int llr_type;
     void *out;
 };
+
+// hi:lo of a * m: four 32 x 32 -> 64-bit multiply-adds (no partial sum overflows).
+__device__ __forceinline__ void mul_wide64(uint64_t a, uint64_t m, uint64_t &hi, uint64_t &lo) {
+    const uint32_t a0 = (uint32_t)a, a1 = (uint32_t)(a >> 32), m0 = (uint32_t)m, m1 = (uint32_t)(m >> 32);
+    const uint64_t p00 = (uint64_t)a0 * m0;
+    const uint64_t p01 = (uint64_t)a0 * m1 + (p00 >> 32);
+    const uint64_t p10 = (uint64_t)a1 * m0 + (uint32_t)p01;
+    hi = (uint64_t)a1 * m1 + (p01 >> 32) + (p10 >> 32);
+    lo = (p10 << 32) | (uint32_t)p00;
+}
 
 __device__ __forceinline__ void philox4x64(uint64_t (&c)[4], uint64_t k0, uint64_t k1) {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        const uint64_t lo0 = 0xD2E7470EE14C6C93ull * c[0], hi0 = __umul64hi(0xD2E7470EE14C6C93ull, c[0]);
-        const uint64_t lo1 = 0xCA5A826395121157ull * c[2], hi1 = __umul64hi(0xCA5A826395121157ull, c[2]);
+        uint64_t lo0, hi0, lo1, hi1;
+        mul_wide64(c[0], 0xD2E7470EE14C6C93ull, hi0, lo0);
+        mul_wide64(c[2], 0xCA5A826395121157ull, hi1, lo1);
         const uint64_t n0 = hi1 ^ c[1] ^ k0, n2 = hi0 ^ c[3] ^ k1;
         c[0] = n0;
         c[1] = lo1;
@@ -51,7 +72,7 @@ __device__ __forceinline__ void philox4x64(uint64_t (&c)[4], uint64_t k0, uint64
 
 __device__ __forceinline__ double unit53(uint64_t x) { return (double)((x >> 11) + 1ull) * 0x1.0p-53; }
 
-// Bits [lo, lo + 16) of the information stream (zero outside [0, n_info)).
+// Bits [lo, lo + 32) of the information stream (zero outside [0, n_info)).
 __device__ __forceinline__ uint32_t info_window(const TxParams &p, int64_t lo) {
     uint32_t v = 0;
 #pragma unroll
@@ -70,63 +91,169 @@ __device__ __forceinline__ uint32_t info_window(const TxParams &p, int64_t lo) {
     return v;
 }
 
-__global__ void transmit_kernel(const TxParams p) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t k0 = 8 * j;
-    if (k0 >= p.n_kept) return;
-    double z[8];
+// Eight normals of blocks 2 j and 2 j + 1, in double precision.
+__device__ __forceinline__ void normals(uint64_t (&w)[2][4], double (&z)[8]) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        uint64_t c[4] = {(uint64_t)(2 * j + h), 0ull, 0ull, 0ull};
-        philox4x64(c, p.seed, p.stream_id);
+    for (int h = 0; h < 2; ++h)
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            const double u = unit53(c[2 * q]), v = unit53(c[2 * q + 1]);
+            const double u = unit53(w[h][2 * q]), v = unit53(w[h][2 * q + 1]);
             const double rad = sqrt(-2.0 * log(u)), ang = 2.0 * 3.14159265358979323846 * v;
             z[4 * h + 2 * q] = rad * cos(ang);
             z[4 * h + 2 * q + 1] = rad * sin(ang);
         }
-    }
-    uint32_t packed = 0;   // 4-bit and hard outputs of this thread's values
+}
+
+// The quantised value of a sample as the bits it has in the output.
+template <int TYPE>
+__device__ __forceinline__ uint32_t quantise(double y, double inv_var2) {
+    if constexpr (TYPE == VD_LLR_S8) return (uint32_t)(int)fmin(fmax(rint(32.0 * y), -127.0), 127.0) & 0xFFu;
+    else if constexpr (TYPE == VD_LLR_S4) return (uint32_t)(int)fmin(fmax(rint(2.0 * y), -7.0), 7.0) & 0xFu;
+    else if constexpr (TYPE == VD_LLR_F16) return (uint32_t)__half_as_ushort(__double2half(y * inv_var2));
+    else return y < 0.0 ? 1u : 0u;
+}
+
+// Double precision for a thread whose values single precision leaves open:
+// eight 16-bit fields.
+template <int TYPE>
+__device__ __noinline__ uint4 exact_values(uint64_t j, uint64_t seed, uint64_t stream_id, uint32_t cbits, double sigma,
+                                           double inv_var2) {
+    uint64_t w[2][4] = {{2 * j, 0ull, 0ull, 0ull}, {2 * j + 1, 0ull, 0ull, 0ull}};
+    philox4x64(w[0], seed, stream_id);
+    philox4x64(w[1], seed, stream_id);
+    double z[8];
+    normals(w, z);
+    uint32_t q[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        const int64_t k = k0 + i;
-        if (k >= p.n_kept) break;
-        const int64_t g = k / p.kept_per_period;
-        const int r = (int)(k - g * p.kept_per_period);
-        const int64_t t = g * p.period + p.pos_phase[r];
-        const int b = p.pos_b[r];
-        const uint32_t reg = info_window(p, t - (p.K - 1)) & ((1u << p.K) - 1u);
-        const uint32_t cbit = (uint32_t)__popc(p.gens[b] & reg) & 1u;
-        const double y = (cbit ? -1.0 : 1.0) + p.sigma * z[i];
-        switch (p.llr_type) {
-        case VD_LLR_S8: {
-            const double q = fmin(fmax(rint(32.0 * y), -127.0), 127.0);
-            static_cast<int8_t *>(p.out)[k] = (int8_t)q;
-            break;
-        }
-        case VD_LLR_S4: {
-            const double q = fmin(fmax(rint(2.0 * y), -7.0), 7.0);
-            packed |= ((uint32_t)(int)q & 0xFu) << (4 * i);
-            break;
-        }
-        case VD_LLR_F16:
-            static_cast<__half *>(p.out)[k] = __double2half(y * p.inv_var2);
-            break;
-        default:   // VD_LLR_HARD
-            packed |= (y < 0.0 ? 1u : 0u) << i;
-            break;
+        const double y = (((cbits >> i) & 1u) ? -1.0 : 1.0) + sigma * z[i];
+        q[i] = quantise<TYPE>(y, inv_var2);
+    }
+    return make_uint4(q[0] | q[1] << 16, q[2] | q[3] << 16, q[4] | q[5] << 16, q[6] | q[7] << 16);
+}
+
+// A Box-Muller pair in single precision.  u = U 2^-53 and v = V 2^-53 enter as
+// integers, so that 1 - u and the angle's offset from the nearest quarter
+// turn are exact before they are rounded to 24 bits.  Errors, with logf,
+// log1pf, sinpif and cospif good to 2 ulp and sqrtf to half of one: ln u
+// 4e-7 of itself (6e-8 of u or 1 - u, at most 1.45 times that in the logarithm, and 2 ulp), rad half of that and
+// 6e-8; the sine and cosine 5e-8 (the angle) and 2.4e-7.  So cos and sin
+// times rad are off by less than 6e-7 rad.
+__device__ __forceinline__ void pair_f32(uint64_t wu, uint64_t wv, float &rad, float &c, float &s) {
+    const uint64_t U = (wu >> 11) + 1ull, V = (wv >> 11) + 1ull;
+    const bool low = U <= (1ull << 52);
+    const float a = __ull2float_rn(low ? U : (1ull << 53) - U) * 0x1.0p-53f;
+    const float ln = low ? logf(a) : log1pf(-a);
+    rad = sqrtf(-2.0f * ln);
+    const uint64_t quad = (V + (1ull << 50)) >> 51;
+    const float r = __ll2float_rn((long long)(V - (quad << 51))) * 0x1.0p-52f;   // half turns, at most 1/4
+    float sn, cs;
+    sincospif(r, &sn, &cs);
+    const bool odd = quad & 1ull;
+    const float x = odd ? sn : cs, y = odd ? cs : sn;
+    c = (quad + 1ull) & 2ull ? -x : x;   // quarter turns 1, 2: negative cosine
+    s = quad & 2ull ? -y : y;            // quarter turns 2, 3: negative sine
+}
+
+template <int TYPE>
+__global__ void __launch_bounds__(256) transmit_kernel(const TxParams p) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t k0 = 8 * j;
+    if (k0 >= p.n_kept) return;
+    // encoder outputs of the thread's kept values: at most eight stages, one window of input bits
+    int64_t g = p.kept_per_period == 1 ? k0 : (int64_t)__umul64hi((uint64_t)k0, p.kpp_magic);
+    int r = (int)(k0 - g * p.kept_per_period);
+    int64_t tg = g * p.period;                        // first stage of the period
+    const int64_t t0 = tg + p.pos_phase[r];
+    const uint32_t win = info_window(p, t0 - (p.K - 1));
+    uint32_t cbits = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int dt = (int)(tg - t0) + p.pos_phase[r];
+        const uint32_t reg = (win >> dt) & ((1u << p.K) - 1u);
+        cbits |= ((uint32_t)__popc(p.gens[p.pos_b[r]] & reg) & 1u) << i;
+        if (++r == p.kept_per_period) {
+            r = 0;
+            tg += p.period;
         }
     }
-    if (p.llr_type == VD_LLR_S4) {
-        // values k0 .. k0+7 are bytes 4j .. 4j+3; the last byte may be partial
-        uint8_t *o = static_cast<uint8_t *>(p.out) + 4 * j;
-        const int64_t nbytes = (p.n_kept + 1) / 2;
+    uint64_t w[2][4] = {{(uint64_t)(2 * j), 0ull, 0ull, 0ull}, {(uint64_t)(2 * j + 1), 0ull, 0ull, 0ull}};
+    philox4x64(w[0], p.seed, p.stream_id);
+    philox4x64(w[1], p.seed, p.stream_id);
+    uint32_t q[8];
+    bool open = false;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            if (4 * j + i < nbytes) o[i] = (uint8_t)(packed >> (8 * i));
-    } else if (p.llr_type == VD_LLR_HARD) {
-        static_cast<uint8_t *>(p.out)[j] = (uint8_t)packed;
+    for (int m = 0; m < 4; ++m) {
+        float rad, cs[2];
+        pair_f32(w[m >> 1][2 * (m & 1)], w[m >> 1][2 * (m & 1) + 1], rad, cs[0], cs[1]);
+        // y = +-1 + sigma z: the pair's error, the rounding of sigma, of the
+        // product and of the sum (2.4e-7 together), each with room to spare
+        const float srad = p.sigma_f * rad, ey = 1.2e-6f * srad + 3e-7f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int i = 2 * m + k;
+            const float y = fmaf(srad, cs[k], ((cbits >> i) & 1u) ? -1.0f : 1.0f);
+            uint32_t lo, hi;
+            if constexpr (TYPE == VD_LLR_S8) {
+                lo = (uint32_t)(int)fminf(fmaxf(rintf(32.0f * (y - ey)), -127.0f), 127.0f) & 0xFFu;
+                hi = (uint32_t)(int)fminf(fmaxf(rintf(32.0f * (y + ey)), -127.0f), 127.0f) & 0xFFu;
+            } else if constexpr (TYPE == VD_LLR_S4) {
+                lo = (uint32_t)(int)fminf(fmaxf(rintf(2.0f * (y - ey)), -7.0f), 7.0f) & 0xFu;
+                hi = (uint32_t)(int)fminf(fmaxf(rintf(2.0f * (y + ey)), -7.0f), 7.0f) & 0xFu;
+            } else if constexpr (TYPE == VD_LLR_F16) {
+                const float x = y * p.inv_var2_f, ex = ey * p.inv_var2_f + 3e-7f * fabsf(x);
+                lo = __half_as_ushort(__float2half_rn(x - ex));
+                hi = __half_as_ushort(__float2half_rn(x + ex));
+            } else {
+                lo = y - ey < 0.0f ? 1u : 0u;
+                hi = y + ey < 0.0f ? 1u : 0u;
+            }
+            q[i] = lo;
+            open |= lo != hi;
+        }
+    }
+    if (open) {
+        const uint4 x = exact_values<TYPE>((uint64_t)j, p.seed, p.stream_id, cbits, p.sigma, p.inv_var2);
+        const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) q[i] = (xs[i >> 1] >> (16 * (i & 1))) & 0xFFFFu;
+    }
+    const int n = p.n_kept - k0 < 8 ? (int)(p.n_kept - k0) : 8;   // values of this thread
+    if constexpr (TYPE == VD_LLR_S8) {
+        int8_t *o = static_cast<int8_t *>(p.out) + k0;
+        if (n == 8 && p.aligned) {
+            *reinterpret_cast<uint2 *>(o) = make_uint2(q[0] | q[1] << 8 | q[2] << 16 | q[3] << 24,
+                                                       q[4] | q[5] << 8 | q[6] << 16 | q[7] << 24);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < n) o[i] = (int8_t)q[i];
+        }
+    } else if constexpr (TYPE == VD_LLR_F16) {
+        uint16_t *o = static_cast<uint16_t *>(p.out) + k0;
+        if (n == 8 && p.aligned) {
+            *reinterpret_cast<uint4 *>(o) =
+                make_uint4(q[0] | q[1] << 16, q[2] | q[3] << 16, q[4] | q[5] << 16, q[6] | q[7] << 16);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (i < n) o[i] = (uint16_t)q[i];
+        }
+    } else {
+        // values past the last one are zero bits (4-bit: two per byte, hard: eight)
+        constexpr int BITS = TYPE == VD_LLR_S4 ? 4 : 1;
+        uint32_t packed = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (i < n) packed |= q[i] << (BITS * i);
+        uint8_t *o = static_cast<uint8_t *>(p.out) + BITS * j;
+        if (BITS == 4 && n == 8 && p.aligned) {
+            *reinterpret_cast<uint32_t *>(o) = packed;
+        } else {
+#pragma unroll
+            for (int i = 0; i < BITS; ++i)
+                if (BITS * n > 8 * i) o[i] = (uint8_t)(packed >> (8 * i));
+        }
     }
 }
 
@@ -185,15 +312,25 @@ extern "C" vd_status vd_transmit(const vd_code *c, const uint32_t *d_bits, int64
             }
     p.sigma = sigma;
     p.inv_var2 = sigma > 0.0 ? 2.0 / (sigma * sigma) : 0.0;
+    p.sigma_f = (float)p.sigma;
+    p.inv_var2_f = (float)p.inv_var2;
+    // k < 2^43, so the rounded-up reciprocal's excess (at most 32 of 2^64) never reaches the quotient
+    if (p.kept_per_period > 1) p.kpp_magic = ~0ull / (uint64_t)p.kept_per_period + 1ull;
+    p.aligned = ((uintptr_t)d_out & 15u) == 0;
     p.seed = seed;
     p.stream_id = stream_id;
-    p.llr_type = llr_type;
     p.out = d_out;
     const int64_t threads = (p.n_kept + 7) / 8;
     const int tb = 256;
     const int64_t blocks = (threads + tb - 1) / tb;
     if (blocks > 0x7FFFFFFF) return fail(VD_EINVAL, "vd_transmit: stream too long");
-    transmit_kernel<<<(unsigned)blocks, tb, 0, (cudaStream_t)stream>>>(p);
+    const cudaStream_t cs = (cudaStream_t)stream;
+    switch (llr_type) {
+    case VD_LLR_S8: transmit_kernel<VD_LLR_S8><<<(unsigned)blocks, tb, 0, cs>>>(p); break;
+    case VD_LLR_S4: transmit_kernel<VD_LLR_S4><<<(unsigned)blocks, tb, 0, cs>>>(p); break;
+    case VD_LLR_F16: transmit_kernel<VD_LLR_F16><<<(unsigned)blocks, tb, 0, cs>>>(p); break;
+    default: transmit_kernel<VD_LLR_HARD><<<(unsigned)blocks, tb, 0, cs>>>(p); break;
+    }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(VD_ECUDA, cudaGetErrorString(e));
     return VD_OK;
