@@ -87,7 +87,8 @@ typedef struct vd_tune {
     int32_t f;         /* frame length (stages decoded per frame) */
     int32_t v;         /* overlap on each side */
     int32_t radix;     /* 2 or 4 */
-    int32_t lanes;     /* threads per pair of frames: 1, 2, 4 (K=7), 4, 8 (K=9); 0 = default */
+    int32_t lanes;     /* threads per pair of frames: 1, 2, 4 (K=7), 4, 8 (K=9); 0 = default.  The
+                          fp16 form is named by 2 (K=7) or 8 (K=9), whatever it takes */
     int32_t threads;   /* threads per block */
     int32_t form;      /* vd_decode kernel form: 0 = by stream length, 1 = persistent
                           (warps pull tasks, interleaved traceback), 2 = one wave */
@@ -176,7 +177,8 @@ vd_status vd_decode_host(const vd_code *code, int n_streams, const void *const *
 /*
  * The configuration vd_decode uses for this code and LLR type when its tune
  * argument is NULL: f, v and radix as given, and the lanes per frame pair and
- * threads per block it picks.  The decoded bits depend only on f, v and the
+ * threads per block it picks (for streams of many frames; few frames take the
+ * other forms of vd_decode).  The decoded bits depend only on f, v and the
  * flags, so this is what a reference decoder needs to reproduce a call.
  * VD_EINVAL on bad arguments, VD_EUNSUPPORTED if there is no kernel.
  */

@@ -1,34 +1,50 @@
-// fp16-LLR / fp32-metric stream kernel instantiations: K=7 with 2 lanes per
-// frame pair, K=9 with 8.
+// fp16-LLR / fp32-metric stream kernel instantiations: a frame pair over 4
+// lanes (K=7), 16 or 8 (K=9).  The caller's names of these forms
+// (vd_tune.lanes) are 2 and 8.
 #include "vd_launch.h"
 #include "vd_stream_f32.cuh"
 
 namespace vd {
 
-cudaError_t launch_stream_f32_k7(int lanes, const StreamParams &p, int64_t blocks, cudaStream_t st) {
-    if (lanes != 2) return cudaErrorInvalidValue;
-    stream_kernel_f32<7, 2, GENS_K7, 2, kThreads><<<(unsigned)blocks, kThreads, 0, st>>>(p);
+namespace {
+
+template <int K> struct F32Of;
+template <> struct F32Of<7> { static constexpr int BETA = 2; static constexpr uint64_t GENS = GENS_K7; };
+template <> struct F32Of<9> { static constexpr int BETA = 3; static constexpr uint64_t GENS = GENS_K9; };
+
+template <int K, int L>
+cudaError_t launch(const StreamParams &p, int64_t blocks, cudaStream_t st) {
+    stream_kernel_f32<K, F32Of<K>::BETA, F32Of<K>::GENS, L, kThreads><<<(unsigned)blocks, kThreads, 0, st>>>(p);
     return cudaGetLastError();
 }
 
-cudaError_t launch_stream_f32_k9(int lanes, const StreamParams &p, int64_t blocks, cudaStream_t st) {
-    if (lanes != 8) return cudaErrorInvalidValue;
-    stream_kernel_f32<9, 3, GENS_K9, 8, kThreads><<<(unsigned)blocks, kThreads, 0, st>>>(p);
-    return cudaGetLastError();
+template <int K, int L>
+F32Geom geom() {
+    using Cfg = StreamCfgF32<K, F32Of<K>::BETA, F32Of<K>::GENS, L>;
+    F32Geom g;
+    g.geom.U = Cfg::U;
+    g.geom.NW = Cfg::NW;
+    g.threads_per_pair = L;
+    return g;
 }
 
-bool geom_f32_k7(int lanes, KernelGeom *g) {
-    if (lanes != 2) return false;
-    g->U = StreamCfgF32<7, 2, GENS_K7, 2>::U;
-    g->NW = StreamCfgF32<7, 2, GENS_K7, 2>::NW;
-    return true;
+}  // namespace
+
+// K=9: 16 lanes per pair while all pairs are resident at once (four blocks
+// of 128 threads an SM), 8 beyond.  Sixteen lanes halve the chain of a stage, eight take 45
+// instructions per frame and stage instead of 62.  Measured (us, 16 / 8 lanes): 2^20 bits
+// 283 / 429, 2^22 (1.7 times the residents) 537 / 490, 2^24 1772 / 1657.  K=7 (4 / 2 lanes):
+// 132 / 201, 166 / 214, 436 / 502.
+F32Geom geom_f32(int K, int64_t n_pairs, int n_sm) {
+    if (K == 7) return geom<7, 4>();
+    return n_pairs * 16 <= (int64_t)n_sm * 4 * kThreads ? geom<9, 16>() : geom<9, 8>();
 }
 
-bool geom_f32_k9(int lanes, KernelGeom *g) {
-    if (lanes != 8) return false;
-    g->U = StreamCfgF32<9, 3, GENS_K9, 8>::U;
-    g->NW = StreamCfgF32<9, 3, GENS_K9, 8>::NW;
-    return true;
+cudaError_t launch_stream_f32(int K, int threads_per_pair, const StreamParams &p, int64_t blocks, cudaStream_t st) {
+    if (K == 7 && threads_per_pair == 4) return launch<7, 4>(p, blocks, st);
+    if (K == 9 && threads_per_pair == 8) return launch<9, 8>(p, blocks, st);
+    if (K == 9 && threads_per_pair == 16) return launch<9, 16>(p, blocks, st);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace vd

@@ -298,7 +298,7 @@ bool geometry(vd::CodeKind kind, int lanes, bool r4, vd::KernelGeom *g) {
 }
 
 struct Plan {
-    int lanes;
+    int lanes, threads_per_pair;
     bool r4;
     bool persistent;   // integer LLRs: the persistent kernel with interleaved traceback
     vd::KernelGeom geom;
@@ -370,8 +370,8 @@ vd_status make_plan(const vd_code *c, int64_t n_info, int f, int v, int radix, u
     } else if (!default_lanes(c->kind, &pl->lanes)) {
         return fail(VD_EUNSUPPORTED, "no kernel for this code");
     }
-    const bool have = f32 ? (c->kind == vd::KIND_K7_R2 ? vd::geom_f32_k7(pl->lanes, &pl->geom)
-                                                       : vd::geom_f32_k9(pl->lanes, &pl->geom))
+    // fp16 input has one form per code, which its callers name by these lanes
+    const bool have = f32 ? pl->lanes == (c->kind == vd::KIND_K7_R2 ? 2 : 8)
                           : geometry(c->kind, pl->lanes, pl->r4, &pl->geom);
     if (!have)
         return fail(VD_EUNSUPPORTED, "no kernel with %d lanes per frame pair (radix %d) for K=%d",
@@ -379,11 +379,17 @@ vd_status make_plan(const vd_code *c, int64_t n_info, int f, int v, int radix, u
     pl->T = n_info + ((flags & VD_TERMINATED) ? c->K - 1 : 0);
     pl->n_win = vd_num_frames(n_info, f);
     pl->n_pairs = (pl->n_win + 1) / 2;
+    pl->threads_per_pair = pl->lanes;
+    if (f32) {
+        const vd::F32Geom g = vd::geom_f32(c->K, pl->n_pairs, sm_count());
+        pl->geom = g.geom;
+        pl->threads_per_pair = g.threads_per_pair;
+    }
     const int64_t wmax = std::min<int64_t>(pl->T, (int64_t)f + 2 * (int64_t)v);
     const int64_t wpad = ((wmax + pl->geom.U - 1) / pl->geom.U) * pl->geom.U;
     if (wpad > (1 << 30)) return fail(VD_EINVAL, "frame too long (%lld stages)", (long long)wmax);
     pl->wpad_max = (int32_t)wpad;
-    const int64_t threads = pl->n_pairs * pl->lanes;
+    const int64_t threads = pl->n_pairs * pl->threads_per_pair;
     pl->n_tasks = (pl->n_pairs + 32 / pl->lanes - 1) / (32 / pl->lanes);
     pl->persistent = false;
     if (!f32) {
@@ -550,11 +556,11 @@ extern "C" vd_status vd_decode(const vd_code *c, const void *d_llr, int llr_type
     }
     switch (c->kind) {
     case vd::KIND_K7_R2:
-        e = f32 ? vd::launch_stream_f32_k7(pl.lanes, p, pl.blocks, cs)
+        e = f32 ? vd::launch_stream_f32(c->K, pl.threads_per_pair, p, pl.blocks, cs)
                 : vd::launch_stream_k7(pl.lanes, pl.r4, p, pl.blocks, cs);
         break;
     case vd::KIND_K9_R3:
-        e = f32 ? vd::launch_stream_f32_k9(pl.lanes, p, pl.blocks, cs)
+        e = f32 ? vd::launch_stream_f32(c->K, pl.threads_per_pair, p, pl.blocks, cs)
                 : vd::launch_stream_k9(pl.lanes, pl.r4, p, pl.blocks, cs);
         break;
     default: return fail(VD_EUNSUPPORTED, "no kernel for this code");

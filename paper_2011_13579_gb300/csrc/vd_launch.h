@@ -56,10 +56,13 @@ constexpr int kSplitWarmup = 16, kSplitGain = 8;
 bool split_plan(int K, const WideParams &in, int n_sm, SplitParams *out, int *ranks, size_t *smem);
 cudaError_t launch_split(int K, const SplitParams &p, int ranks, size_t smem, cudaStream_t st);
 
-cudaError_t launch_stream_f32_k7(int lanes, const StreamParams &p, int64_t blocks, cudaStream_t st);
-cudaError_t launch_stream_f32_k9(int lanes, const StreamParams &p, int64_t blocks, cudaStream_t st);
-bool geom_f32_k7(int lanes, KernelGeom *g);
-bool geom_f32_k9(int lanes, KernelGeom *g);
+// fp16 input: kernel shape for a stream of n_pairs frame pairs, and its launch.
+struct F32Geom {
+    KernelGeom geom;
+    int threads_per_pair;
+};
+F32Geom geom_f32(int K, int64_t n_pairs, int n_sm);
+cudaError_t launch_stream_f32(int K, int threads_per_pair, const StreamParams &p, int64_t blocks, cudaStream_t st);
 bool geom_k7(int lanes, bool radix4, KernelGeom *g);
 bool geom_k9(int lanes, bool radix4, KernelGeom *g);
 
