@@ -118,15 +118,14 @@ int vd_code_supported(int K, int beta, const uint32_t *gens_octal);
 
 /*
  * Segmented (or full-length) stream decode, Algorithms 1-2 over the frames
- * of Sec. III.  Long int8 / 4-bit streams (at least one task of frame pairs
- * per resident warp) run a persistent kernel whose warps pull tasks and trace
- * one task back while decoding the next forward; shorter ones a kernel with
- * one frame pair per lane group (tune->form overrides).  Streams of few frames
- * run, unless tune asks for lanes or a form, a kernel that spreads each frame
- * pair over a quarter warp (K=7) or a warp (K=9) and keeps its survivors in
- * shared memory; few long frames are decoded in overlapping segments at once,
- * which run again until their metrics agree with those of the frame decoded in
- * one piece.  All give the same bits.
+ * of Sec. III.  Unless tune asks for lanes or a form, the kernel goes by the
+ * stream: few long frames are decoded in overlapping segments at once, which
+ * run again until their metrics agree with those of the frame decoded in
+ * one piece; few frames spread each frame pair over a quarter warp (K=7) or a
+ * warp (K=9); both keep their survivors in shared memory.  Longer streams take a
+ * kernel with one lane group per frame pair, or a persistent one whose warps
+ * pull tasks and trace one task back while decoding the next forward.  All
+ * give the same bits.
  *   d_llr:    device pointer to the received LLRs of the whole stream, of
  *             llr_type, in transmitted order (kept positions only when the
  *             code is punctured): n_kept(T) values, T = n_info (+K-1 if
@@ -135,7 +134,8 @@ int vd_code_supported(int K, int beta, const uint32_t *gens_octal);
  *   f, v:     frame length and overlap; f must be a multiple of 32 unless
  *             f >= n_info (a single frame).  v >= 0.  A full-length decode is
  *             f >= n_info with v >= K-1.
- *   radix:    2 or 4 (same bits either way).
+ *   radix:    2 or 4 (same bits either way; unless tune asks for lanes or a
+ *             form, the library runs the steps that are faster).
  *   flags:    VD_TERMINATED, VD_START_UNKNOWN.
  *   d_out:    device pointer to ceil(n_info/32) uint32 words (written).
  *   d_pm:     NULL, or device pointer to n_frames x 2^(K-1) int32 receiving
@@ -569,9 +569,9 @@ int64_t vd_num_frames(int64_t n_info, int f);
 int64_t vd_num_kept(const vd_code *code, int64_t T);
 
 /* Bytes of survivor scratch one stream decode needs (informational, int8
- * LLRs).  A stream with at least one task of frame pairs per resident warp
- * of the persistent kernel needs a fixed two buffers per resident warp; a
- * shorter one needs one buffer per frame pair's lane group. */
+ * LLRs): none where the survivors stay in shared memory (few frames), a
+ * buffer per frame pair's lane group otherwise, a fixed two buffers per resident
+ * warp for the persistent kernel; and the depunctured copy of a punctured code's values. */
 int64_t vd_scratch_bytes(const vd_code *code, int64_t n_info, int f, int v, int radix,
                          const vd_tune *tune);
 

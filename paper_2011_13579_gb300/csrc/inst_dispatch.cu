@@ -60,6 +60,13 @@ cudaError_t stream_persistent_occupancy(int K, int lanes, bool radix4, int *bloc
     return cudaErrorInvalidValue;
 }
 
+cudaError_t stream_wave_occupancy(int K, int lanes, bool radix4, int *blocks_per_sm) {
+#define X(KK, R4, L) if (K == KK && radix4 == R4 && lanes == L) return occupancy_wave_v<KK, R4, L>(blocks_per_sm);
+    VD_VARIANT_LIST(X)
+#undef X
+    return cudaErrorInvalidValue;
+}
+
 bool geom_k7(int lanes, bool radix4, KernelGeom *g) {
 #define X(K, R4, L)                                                        \
     if (K == 7 && radix4 == R4 && lanes == L) {                            \

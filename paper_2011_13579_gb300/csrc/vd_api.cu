@@ -297,30 +297,24 @@ bool geometry(vd::CodeKind kind, int lanes, bool r4, vd::KernelGeom *g) {
     }
 }
 
+// How a stream is decoded: few long frames in segments, few frames each over
+// many lanes, one lane group per frame pair, or (integer LLRs) resident warps that pull tasks.
+enum class Form { SPLIT, WIDE, WAVE, PERSISTENT };
+
 struct Plan {
+    Form form;
     int lanes, threads_per_pair;
     bool r4;
-    bool persistent;   // integer LLRs: the persistent kernel with interleaved traceback
     vd::KernelGeom geom;
     int64_t T, n_win, n_pairs, n_tasks, blocks;
     int32_t wpad_max;
-    size_t surv_bytes;
+    size_t surv_bytes;         // 0 where the survivors stay in shared memory
+    vd::SplitParams split;     // SPLIT (without pointers)
+    vd::WideParams wide;       // WIDE (without pointers)
+    int ranks;                 // SPLIT: blocks per frame
+    bool wide_full;            // WIDE: a whole warp's pairs per block
+    size_t smem;               // SPLIT, WIDE
 };
-
-// Streams with at least this many tasks per resident warp take the persistent
-// form (measured on GB300: below one wave the one-pair-per-lane-group kernel
-// is faster, from one wave up the persistent one, for K=7 and K=9).
-constexpr int64_t kPersistentWaves = 1;
-
-// Streams of few frames take the wide form (vd_wide.cuh) while its blocks
-// make at most this many waves of what the SMs hold at once (shared memory
-// bounds that).  Both forms' times grow with the frame length and no other
-// form gets faster below one of its own waves, so the line is a number of
-// waves.  Measured (GB300, us per call, wide / otherwise): K=7, f = 256:
-// 10^5 bits 22 / 101, 10^6 23 / 97, 4.2 M (1.9 waves) 56 / 98, 8.4 M (3.9) 103 / 106, 16.8 M
-// 193 / 167; K=9, f = 512: 10^5 bits 44 / 335, 10^6 (1.3) 83 / 335, 4.2 M (5.4)
-// 261 / 346, 8.4 M (10.8) 500 / 360.
-constexpr double kWideWavesK7 = 3.5, kWideWavesK9 = 7.0;
 
 int sm_count() {
     static std::mutex mu;
@@ -335,28 +329,77 @@ int sm_count() {
     return cache[dev] = n;
 }
 
-bool take_wide(int K, int64_t blocks, size_t smem) {
-    const int64_t per_sm = (int64_t)((228u * 1024u) / (smem + 1024u));   // 228 KB an SM, 1 KB of it reserved per block
-    return (double)blocks <= (K == 7 ? kWideWavesK7 : kWideWavesK9) * (double)(sm_count() * std::max<int64_t>(1, per_sm));
-}
-
-// Resident blocks per SM of the persistent stream kernel, per device and shape.
-int persistent_blocks_per_sm(int K, int lanes, bool r4) {
+// Resident blocks per SM of the persistent or the one-wave stream kernel, per device and shape.
+int blocks_per_sm(bool persistent, int K, int lanes, bool r4) {
     static std::mutex mu;
-    static std::map<std::tuple<int, int, int, int>, int> cache;
+    static std::map<std::tuple<int, bool, int, int, bool>, int> cache;
     int dev = 0;
     cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lk(mu);
-    const auto key = std::make_tuple(dev, K, lanes, (int)r4);
+    const auto key = std::make_tuple(dev, persistent, K, lanes, r4);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     int bps = 0;
-    if (vd::stream_persistent_occupancy(K, lanes, r4, &bps) != cudaSuccess) {
+    if ((persistent ? vd::stream_persistent_occupancy(K, lanes, r4, &bps)
+                    : vd::stream_wave_occupancy(K, lanes, r4, &bps)) != cudaSuccess) {
         cudaGetLastError();
         bps = 0;
     }
     cache[key] = bps;
     return bps;
+}
+
+// The wide form, while its blocks make at most this many waves of what the SMs
+// hold at once (shared memory bounds that): all forms' times grow with the
+// frame length, and no other form gets faster below one of its own waves.  Measured
+// (GB300, us per call, wide / the next form): K=7, f = 256: 10^5 bits 22 / 64, 10^6 23 / 60,
+// 4.2 M (1.9 waves) 56 / 67, 8.4 M (3.9) 103 / 99; K=9, f = 512: 10^5 bits 44 / 136,
+// 10^6 (1.3) 83 / 136, 2.1 M (2.6) 130 / 136, 3 M (3.9) 199 / 188.
+constexpr double kWideWavesK7 = 3.5, kWideWavesK9 = 2.6;
+
+bool take_wide(int K, int64_t blocks, size_t smem) {
+    const int64_t per_sm = (int64_t)((228u * 1024u) / (smem + 1024u));   // 228 KB an SM, 1 KB of it reserved per block
+    return (double)blocks <= (K == 7 ? kWideWavesK7 : kWideWavesK9) * (double)(sm_count() * std::max<int64_t>(1, per_sm));
+}
+
+size_t wave_scratch(int64_t n_pairs, int lanes, int64_t wmax, const vd::KernelGeom &g, int64_t *blocks) {
+    *blocks = (n_pairs * lanes + vd::kThreads - 1) / vd::kThreads;
+    return (size_t)*blocks * vd::kThreads * (size_t)((wmax + g.U - 1) / g.U * g.U) * g.NW * 4u;
+}
+
+// Lanes per pair and form of a stream too long for the forms above, when the
+// caller leaves both open (us per call at the stated bits, f = 256 or 512).
+// K=7: two lanes per pair while all pairs are resident (10 M: 132 against 157
+// with one); one lane while no scheduler has more than two warps (16.8 M: 159
+// against 187); then the persistent form (20 M: 217 against 241).
+// K=9: eight lanes while all pairs are resident (4.2 M: 188 against 283 with four), then four
+// while they are (8.4 M: 314 against 362), then eight again (10 M 437 / 532,
+// 16.8 M 590 / 621, 20 M 739 / 801 against the persistent form with four) while
+// the survivors of all pairs take no more memory than the persistent form's.
+void choose_shape(const vd_code *c, bool r4, int64_t n_pairs, int64_t wmax, int *lanes, Form *form) {
+    const int64_t n_sm = sm_count();
+    auto resident_pairs = [&](int l) { return n_sm * blocks_per_sm(false, c->K, l, r4) * (vd::kThreads / l); };
+    if (c->kind == vd::KIND_K7_R2) {
+        *lanes = n_pairs <= resident_pairs(2) ? 2 : 1;
+        *form = *lanes == 2 || (n_pairs + 31) / 32 <= 2 * 4 * n_sm ? Form::WAVE : Form::PERSISTENT;
+        return;
+    }
+    *form = Form::WAVE;
+    *lanes = 8;
+    if (n_pairs <= resident_pairs(8)) return;
+    if (n_pairs <= resident_pairs(4)) {
+        *lanes = 4;
+        return;
+    }
+    vd::KernelGeom g8, g4;
+    int64_t blocks = 0;
+    if (!geometry(c->kind, 8, r4, &g8) || !geometry(c->kind, 4, r4, &g4)) return;
+    const size_t persistent = 2u * (size_t)(n_sm * blocks_per_sm(true, c->K, 4, r4)) * vd::kThreads *
+                              (size_t)((wmax + g4.U - 1) / g4.U * g4.U) * g4.NW * 4u;
+    if (wave_scratch(n_pairs, 8, wmax, g8, &blocks) > persistent) {
+        *lanes = 4;
+        *form = Form::PERSISTENT;
+    }
 }
 
 vd_status make_plan(const vd_code *c, int64_t n_info, int f, int v, int radix, uint32_t flags,
@@ -371,48 +414,64 @@ vd_status make_plan(const vd_code *c, int64_t n_info, int f, int v, int radix, u
         return fail(VD_EUNSUPPORTED, "no kernel for this code");
     }
     // fp16 input has one form per code, which its callers name by these lanes
-    const bool have = f32 ? pl->lanes == (c->kind == vd::KIND_K7_R2 ? 2 : 8)
-                          : geometry(c->kind, pl->lanes, pl->r4, &pl->geom);
-    if (!have)
+    if (f32 ? pl->lanes != (c->kind == vd::KIND_K7_R2 ? 2 : 8) : !geometry(c->kind, pl->lanes, pl->r4, &pl->geom))
         return fail(VD_EUNSUPPORTED, "no kernel with %d lanes per frame pair (radix %d) for K=%d",
                     pl->lanes, radix, c->K);
     pl->T = n_info + ((flags & VD_TERMINATED) ? c->K - 1 : 0);
     pl->n_win = vd_num_frames(n_info, f);
     pl->n_pairs = (pl->n_win + 1) / 2;
-    pl->threads_per_pair = pl->lanes;
+    const int64_t wmax = std::min<int64_t>(pl->T, (int64_t)f + 2 * (int64_t)v);
+    if (wmax > (1 << 30)) return fail(VD_EINVAL, "frame too long (%lld stages)", (long long)wmax);
+    pl->form = Form::WAVE;
+    pl->surv_bytes = 0;
+    const int form = tune ? tune->form : 0;
     if (f32) {
         const vd::F32Geom g = vd::geom_f32(c->K, pl->n_pairs, sm_count());
         pl->geom = g.geom;
         pl->threads_per_pair = g.threads_per_pair;
+    } else if ((!tune || tune->lanes == 0) && form == 0) {   // the library's choice
+        vd::WideParams wp;
+        memset(&wp, 0, sizeof wp);
+        wp.n_info = n_info;
+        wp.T = pl->T;
+        wp.f = f;
+        wp.v = v;
+        wp.n_win = pl->n_win;
+        wp.n_pairs = pl->n_pairs;
+        wp.flags = flags;
+        if (vd::split_plan(c->K, wp, sm_count(), &pl->split, &pl->ranks, &pl->smem)) {
+            pl->form = Form::SPLIT;
+            return VD_OK;
+        }
+        if (vd::wide_plan(c->K, wp, &pl->wide, &pl->blocks, &pl->smem, &pl->wide_full) &&
+            take_wide(c->K, pl->blocks, pl->smem)) {
+            pl->form = Form::WIDE;
+            return VD_OK;
+        }
+        // K=7 radix 4 takes radix-2 steps here (the same bits): us, radix-4 / radix-2
+        // kernels: 10 M bits 145 / 131, 16.8 M 183 / 159, 67 M 567 / 481
+        if (c->kind == vd::KIND_K7_R2) pl->r4 = false;
+        choose_shape(c, pl->r4, pl->n_pairs, wmax, &pl->lanes, &pl->form);
+        geometry(c->kind, pl->lanes, pl->r4, &pl->geom);
+        pl->threads_per_pair = pl->lanes;
+    } else {
+        // the caller's lanes; the persistent form from a task per resident warp up
+        pl->threads_per_pair = pl->lanes;
+        const int64_t tasks = (pl->n_pairs + 32 / pl->lanes - 1) / (32 / pl->lanes);
+        const int64_t warps = (int64_t)sm_count() * blocks_per_sm(true, c->K, pl->lanes, pl->r4) * (vd::kThreads / 32);
+        if (warps > 0 && (form == 1 || (form == 0 && tasks >= warps))) pl->form = Form::PERSISTENT;
     }
-    const int64_t wmax = std::min<int64_t>(pl->T, (int64_t)f + 2 * (int64_t)v);
     const int64_t wpad = ((wmax + pl->geom.U - 1) / pl->geom.U) * pl->geom.U;
     if (wpad > (1 << 30)) return fail(VD_EINVAL, "frame too long (%lld stages)", (long long)wmax);
     pl->wpad_max = (int32_t)wpad;
-    const int64_t threads = pl->n_pairs * pl->threads_per_pair;
     pl->n_tasks = (pl->n_pairs + 32 / pl->lanes - 1) / (32 / pl->lanes);
-    pl->persistent = false;
-    if (!f32) {
-        // Long streams (a task per resident warp or more): resident warps
-        // pull tasks and hide each task's traceback behind the next task's
-        // forward pass; each owns two survivor buffers.  Shorter streams are
-        // less than one wave of warps, for which the one-pair-per-lane-group
-        // kernel is faster.
-        int n_sm = 0, dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-        const int bps = persistent_blocks_per_sm(c->K, pl->lanes, pl->r4);
-        const int64_t resident_warps = (int64_t)n_sm * bps * (vd::kThreads / 32);
-        const int form = tune ? tune->form : 0;
-        if (bps >= 1 && (form == 1 || (form == 0 && pl->n_tasks >= kPersistentWaves * resident_warps))) {
-            pl->persistent = true;
-            pl->blocks = (int64_t)n_sm * bps;
-            pl->surv_bytes = 2u * (size_t)pl->blocks * vd::kThreads * (size_t)wpad * pl->geom.NW * 4u;
-        }
-    }
-    if (!pl->persistent) {
-        pl->blocks = (threads + vd::kThreads - 1) / vd::kThreads;
-        pl->surv_bytes = (size_t)pl->blocks * vd::kThreads * (size_t)wpad * pl->geom.NW * 4u;
+    if (pl->form == Form::PERSISTENT) {
+        // resident warps pull tasks and hide each task's traceback behind the
+        // next task's forward pass; each owns two survivor buffers
+        pl->blocks = (int64_t)sm_count() * blocks_per_sm(true, c->K, pl->lanes, pl->r4);
+        pl->surv_bytes = 2u * (size_t)pl->blocks * vd::kThreads * (size_t)wpad * pl->geom.NW * 4u;
+    } else {
+        pl->surv_bytes = wave_scratch(pl->n_pairs, pl->threads_per_pair, wmax, pl->geom, &pl->blocks);
     }
     return VD_OK;
 }
@@ -487,33 +546,21 @@ extern "C" vd_status vd_decode(const vd_code *c, const void *d_llr, int llr_type
         llr = (const int8_t *)buf;
     }
 
-    if (!f32 && (!tune || (tune->lanes == 0 && tune->form == 0))) {   // the library's choice
-        vd::WideParams wp, wide;
-        wp.llr = llr;
-        wp.n_info = n_info;
-        wp.T = pl.T;
-        wp.f = f;
-        wp.v = v;
-        wp.n_win = pl.n_win;
-        wp.n_pairs = pl.n_pairs;
-        wp.flags = flags;
-        wp.out = d_out;
-        wp.pm_out = d_pm;
-        int64_t blocks = 0;
-        size_t smem = 0;
-        bool full = false;
-        vd::SplitParams sp;
-        int ranks = 0;
-        if (vd::split_plan(c->K, wp, sm_count(), &sp, &ranks, &smem)) {
-            const cudaError_t e = vd::launch_split(c->K, sp, ranks, smem, cs);
-            if (e != cudaSuccess) return cuda_fail(e, "decode launch");
-            return VD_OK;
+    if (pl.form == Form::SPLIT || pl.form == Form::WIDE) {
+        if (pl.form == Form::SPLIT) {
+            pl.split.llr = llr;
+            pl.split.out = d_out;
+            pl.split.pm_out = d_pm;
+        } else {
+            pl.wide.llr = llr;
+            pl.wide.out = d_out;
+            pl.wide.pm_out = d_pm;
         }
-        if (vd::wide_plan(c->K, wp, &wide, &blocks, &smem, &full) && take_wide(c->K, blocks, smem)) {
-            const cudaError_t e = vd::launch_wide(c->K, wide, blocks, smem, full, cs);
-            if (e != cudaSuccess) return cuda_fail(e, "decode launch");
-            return VD_OK;
-        }
+        const cudaError_t e = pl.form == Form::SPLIT
+                                  ? vd::launch_split(c->K, pl.split, pl.ranks, pl.smem, cs)
+                                  : vd::launch_wide(c->K, pl.wide, pl.blocks, pl.smem, pl.wide_full, cs);
+        if (e != cudaSuccess) return cuda_fail(e, "decode launch");
+        return VD_OK;
     }
 
     void *surv = nullptr;
@@ -543,7 +590,7 @@ extern "C" vd_status vd_decode(const vd_code *c, const void *d_llr, int llr_type
     if (pl.blocks > 0x7FFFFFFF) return fail(VD_EINVAL, "stream too long for one launch");
     cudaError_t e;
     p.llr_bytes = pl.T * c->beta * (f32 ? 2 : 1);
-    if (pl.persistent) {
+    if (pl.form == Form::PERSISTENT) {
         void *ctr = nullptr;
         st = get_scratch(3, 256, cs, &ctr);
         if (st != VD_OK) return st;

@@ -4,36 +4,18 @@
 //   * a register holds the path metrics of ONE state for TWO frames, as the
 //     two 16-bit halves (frame 0 low, frame 1 high).  Every add-compare-select
 //     is then a pure 16x2 SIMD instruction; the two frames never interact.
-//   * metrics live in unsigned 16-bit halves.  Every N stages they are
-//     normalised: subtract the metric of state 0, add F + S, clamp below at F.
-//     S = (K-1)(delta_max - delta_min) + 1 bounds the spread of live metrics
-//     (and is the head start given to state 0 of a frame that starts from the
-//     reset state), B = beta * 127 bounds |branch metric| and F = (N+1) B.
-//     Between normalisations a metric moves by at most B per stage, so every
-//     metric and every candidate metric + branch metric stays in [0, 32767]
-//     and the packed 16-bit additions and maxima are exact.  Subtracting a
+//   * a half holds 2^ES m + j, unsigned: m the path metric, kept small by a
+//     per-chunk shift (StreamCfg), and j < 2^ES the decisions of the current
+//     record of ES stages along the state's survivor (Eq. SP0: 1 = the odd predecessor p1 =
+//     2f+1 wins, ties included, as Algorithm 1's strict ">" gives).  The odd
+//     candidate of stage k of a record carries + 2^k, so the max itself sets bit k
+//     exactly when the odd predecessor wins or ties and carries the winner's
+//     lower bits along; the fields are stored and cleared after the record.  Branch
+//     metrics are biased to be non-negative, so every metric and every candidate stays in
+//     [0, 65535] and the packed 16-bit additions and maxima are exact.  Subtracting a
 //     per-stage constant from every metric changes no decision (Eq. PM is
-//     invariant under it); the clamp only touches states that are not
-//     reachable from the known start state, whose candidates lose every
-//     comparison anyway, and it is gone after K-1 stages.
-//   * the decision bit of Eq. SP0 (1 = the odd predecessor p1 = 2f+1 wins,
-//     ties included, as Algorithm 1's strict ">" gives) is bit 15 / bit 31 of
-//     the 32-bit sum  c_odd - c_even + 0x8000 (per half), which one 3-input
-//     integer add computes without carries crossing the halves.
-//   * embedded form (radix-2 K=7): a half holds 8 m + j, where the three
-//     low bits j are the decisions of the current group of three stages
-//     along the state's survivor.  The odd candidate of stage k of the group
-//     carries + 2^k, so the max itself sets bit k exactly when the odd
-//     predecessor wins or ties and carries the winner's lower bits along;
-//     the fields are stored and cleared after the group.  Every chunk of
-//     U = 6 stages starts by subtracting the minimum over the states down to
-//     the floor F = U B (folded into the branch metrics of its first stage,
-//     no clamp), and a frame that starts from the reset state gets the
-//     code's tight head start HT (Code::HT) instead of S; the bound is
-//     8 (F + HT + (2 (K-2) + U) B) + 7 <= 65535 (see StreamCfg).  A two-stage
-//     form (4 m + j, state 0 as the reference every N = 18 stages, bound
-//     4 (F + 2S + (N+1) B) + 3 <= 65535) serves codes where three stages do
-//     not fit.
+//     invariant under it).  A frame that starts from the reset state gets the
+//     code's head start HT on state 0 (Code::HT) in place of minus infinity elsewhere.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>

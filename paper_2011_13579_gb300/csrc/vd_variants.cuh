@@ -12,12 +12,6 @@ template <int K> struct CodeOf;
 template <> struct CodeOf<7> { static constexpr int BETA = 2; static constexpr uint64_t GENS = GENS_K7; };
 template <> struct CodeOf<9> { static constexpr int BETA = 3; static constexpr uint64_t GENS = GENS_K9; };
 
-template <int K, bool R4, int L>
-cudaError_t launch_stream_v(const StreamParams &p, int64_t blocks, cudaStream_t st) {
-    stream_kernel<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads><<<(unsigned)blocks, kThreads, 0, st>>>(p);
-    return cudaGetLastError();
-}
-
 // Dynamic shared memory of the persistent kernels (PersistentSmem).  A
 // block may use more than 48 KB only after the kernel opts in, once per
 // device (the attribute belongs to the kernel in that device's context);
@@ -38,6 +32,27 @@ cudaError_t opt_in_smem(Kern kern, size_t bytes, std::atomic<uint64_t> &done) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e == cudaSuccess && bit) done.fetch_or(bit, std::memory_order_acq_rel);
     return e;
+}
+
+template <int K, bool R4, int L>
+cudaError_t launch_stream_v(const StreamParams &p, int64_t blocks, cudaStream_t st) {
+    constexpr size_t bytes = StreamSmem<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads>::BYTES;
+    static std::atomic<uint64_t> done{0};
+    const cudaError_t e = opt_in_smem(stream_kernel<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads>, bytes, done);
+    if (e != cudaSuccess) return e;
+    stream_kernel<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads>
+        <<<(unsigned)blocks, kThreads, bytes, st>>>(p);
+    return cudaGetLastError();
+}
+
+template <int K, bool R4, int L>
+cudaError_t occupancy_wave_v(int *blocks_per_sm) {
+    constexpr size_t bytes = StreamSmem<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads>::BYTES;
+    static std::atomic<uint64_t> done{0};
+    const auto kern = stream_kernel<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads>;
+    const cudaError_t e = opt_in_smem(kern, bytes, done);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, kThreads, bytes);
 }
 
 template <int K, bool R4, int L>
@@ -112,6 +127,7 @@ cudaError_t occupancy_stream_v(int *blocks_per_sm) {
 
 #define VD_DECLARE_VARIANT(K, R4, L)                                                           \
     extern template cudaError_t launch_stream_v<K, R4, L>(const StreamParams &, int64_t, cudaStream_t); \
+    extern template cudaError_t occupancy_wave_v<K, R4, L>(int *);                              \
     extern template cudaError_t launch_batch_v<K, R4, L>(const BatchParams &, int64_t, cudaStream_t);   \
     extern template cudaError_t occupancy_v<K, R4, L>(int *);                                   \
     extern template cudaError_t launch_stream_persistent_v<K, R4, L>(const StreamParams &, int64_t, \

@@ -81,3 +81,24 @@ def check(K, code, oc, beta, shapes, term, unknown, kind, rng):
         assert np.array_equal(out.cpu().numpy().view(np.uint32), ow), (n, f, v)
         whole = [min(T, (s + 1) * f + v) - max(0, s * f - v) >= K - 1 for s in range(pm.shape[0])]
         assert np.array_equal(pm.cpu().numpy()[whole].astype(np.int64), opm[whole]), (n, f, v)
+
+
+@pytest.mark.parametrize("K,lanes,sizes", [(7, 1, (3_000_001, 9_000_000, 16_000_007, 21_000_000)),
+                                           (9, 4, (1_500_001, 3_000_000, 9_000_000, 12_000_001, 21_000_000))])
+def test_every_choice_of_form_gives_the_same_bits(K, lanes, sizes):
+    """Streams on each side of the lines between the forms: what the library
+    chooses, for either radix, against the one-wave kernel with the lanes named."""
+    rng = np.random.Generator(np.random.PCG64(950 + K))
+    code, beta = vd.Code(K, GENS[K]), len(GENS[K])
+    f, v = (256, 42) if K == 7 else (512, 64)
+    q = torch.from_numpy(synth.make_stream(rng, K, GENS[K], 1 << 20, 2.0, False).s8().view(np.uint8)).cuda()
+    q = q.repeat(sizes[-1] // (1 << 20) + 1)      # one received stretch over and over: a codeword but at the seams
+    tune = vd.VdTune()
+    tune.lanes, tune.form = lanes, 2
+    for n in sizes:
+        outs = [torch.full(((n + 31) // 32,), -1, dtype=torch.int32, device="cuda") for _ in range(3)]
+        vd.vd_decode(code.handle, q[:beta * n], vd.VD_LLR_S8, n, f, v, 2, vd.VD_START_UNKNOWN, outs[0], None, tune)
+        for radix, out in ((2, outs[1]), (4, outs[2])):
+            vd.vd_decode(code.handle, q[:beta * n], vd.VD_LLR_S8, n, f, v, radix, vd.VD_START_UNKNOWN, out)
+        vd.vd_sync()
+        assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2]), n
