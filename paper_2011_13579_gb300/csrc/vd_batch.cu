@@ -496,6 +496,8 @@ extern "C" vd_status vd_batch_plan_create(vd_batch_plan **out, const vd_code *co
     cudaError_t e = cudaMalloc((void **)&pl->d_counters, 64 * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc((void **)&pl->d_status, 64 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(pl->d_status, 0, 64 * sizeof(int), cs);
+    // a chained launch, which may be the first, takes the counters as it finds them
+    if (e == cudaSuccess) e = cudaMemsetAsync(pl->d_counters, 0, 64 * sizeof(int), cs);
     if (e != cudaSuccess) { free_plan(pl); return cuda_fail(e, "plan counters"); }
     e = cudaStreamSynchronize(cs);   // host vectors above go out of scope
     if (e != cudaSuccess) { free_plan(pl); return cuda_fail(e, "cudaStreamSynchronize"); }
