@@ -96,6 +96,8 @@ def build(force: bool = False) -> str:
 def lib():
     """The loaded libvd.so; raises if it has not been built."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -347,12 +349,15 @@ def vd_release_scratch() -> None:
 
 
 def _stream_handle(stream):
+    """The cudaStream_t as an int.  Short decodes are bound by this binding
+    (21 us a call with stream objects, pointer objects and a view per call, on the
+    GB300's host), so the current stream is read without making an object of it."""
     if stream is None:
         import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-    if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        if torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        return torch.cuda.current_stream().cuda_stream
+    return stream if isinstance(stream, int) else stream.cuda_stream
 
 
 def vd_decode(handle, llr, llr_type, n_info, f, v, radix, flags, out, pm=None, tune=None, stream=None):
@@ -363,12 +368,12 @@ def vd_decode(handle, llr, llr_type, n_info, f, v, radix, flags, out, pm=None, t
             raise ValueError(f"{name} must be a CUDA tensor")
         if t is not None and not t.is_contiguous():
             raise ValueError(f"{name} must be contiguous")
-    _check(lib().vd_decode(ctypes.c_void_p(handle), ctypes.c_void_p(llr.data_ptr()), int(llr_type),
-                           int(n_info), int(f), int(v), int(radix), int(flags),
-                           ctypes.c_void_p(out.data_ptr()),
-                           ctypes.c_void_p(pm.data_ptr()) if pm is not None else None,
-                           ctypes.byref(tune) if tune is not None else None,
-                           _stream_handle(stream)))
+    # the argument types convert plain ints and None
+    status = lib().vd_decode(handle, llr.data_ptr(), int(llr_type), int(n_info), int(f), int(v), int(radix),
+                             int(flags), out.data_ptr(), pm.data_ptr() if pm is not None else None,
+                             ctypes.byref(tune) if tune is not None else None, _stream_handle(stream))
+    if status != VD_OK:
+        _check(status)
 
 
 def vd_decode_noalloc(handle, llr, n_info, f, v, radix, flags, out, stream=None):
@@ -676,4 +681,6 @@ def decode(code: Code, llr, n_info, f, v, radix=2, terminated=False, start_unkno
         tune = VdTune()
         tune.lanes = int(lanes)
     vd_decode(code.handle, llr, llr_type, n_info, f, v, radix, flags, out, pm, tune, stream)
-    return (out[:nw], pm) if want_pm else out[:nw]
+    if out.dim() != 1 or out.shape[0] != nw:
+        out = out[:nw]
+    return (out, pm) if want_pm else out
