@@ -261,18 +261,23 @@ struct PrepParams {
     const uint8_t *src;       // kept values: int8, or 4-bit packed (two per byte)
     int64_t n_kept;           // number of kept values available
     int64_t T;                // stages to produce
-    int beta, period, kept_per_period, llr_type;
-    uint8_t punct[4][8];
-    int kept_prefix[9];
+    int beta, llr_type;
+    vd::PrepTable table;
+    int64_t piece_words;      // output words of a block's piece (whole cycles)
     int8_t *dst;              // [T][beta]
 };
 
 // Expands the transmitted values of each stage to beta int8 LLRs, with 0 at
 // erased positions (depuncturing) and 4-bit values sign-extended
-// (vd_prep.cuh); a grid-stride loop over whole puncturing periods.
-__global__ void prep_kernel(const PrepParams p) {
-    vd::prep_expand(p.src, 0, p.n_kept, p.llr_type, p.T, p.beta, p.period, p.kept_per_period, p.punct, p.dst,
-                    (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
+// (vd_prep.cuh); a grid-stride loop over pieces of output words.
+__global__ void __launch_bounds__(256) prep_kernel(const __grid_constant__ PrepParams p) {
+    const int64_t bytes = p.T * p.beta, kept = p.piece_words / p.table.words * p.table.kept;
+    for (int64_t i = blockIdx.x; 4 * i * p.piece_words < bytes; i += gridDim.x) {
+        const int64_t at = 4 * i * p.piece_words, left = bytes - at;
+        vd::prep_piece(p.src, i * kept, p.n_kept, p.llr_type,
+                       (uint32_t)(left < 4 * p.piece_words ? left : 4 * p.piece_words), p.table, p.dst + at, threadIdx.x,
+                       blockDim.x);
+    }
 }
 
 }  // namespace
@@ -531,15 +536,13 @@ extern "C" vd_status vd_decode(const vd_code *c, const void *d_llr, int llr_type
         pp.n_kept = vd_num_kept(c, pl.T);
         pp.T = pl.T;
         pp.beta = c->beta;
-        pp.period = c->period;
-        pp.kept_per_period = c->kept_per_period;
         pp.llr_type = llr_type;
-        memcpy(pp.punct, c->punct, sizeof pp.punct);
-        memcpy(pp.kept_prefix, c->kept_prefix, sizeof pp.kept_prefix);
+        pp.table = vd::prep_table(c->beta, c->period, c->punct);
         pp.dst = (int8_t *)buf;
         const int tb = 256;
-        const int64_t groups = (pl.T + c->period - 1) / c->period;
-        const int64_t blocks = std::min<int64_t>((groups + tb - 1) / tb, 4096);
+        pp.piece_words = vd::prep_piece_words(pp.table, 4 * tb);
+        const int64_t words = (pl.T * c->beta + 3) / 4;
+        const int64_t blocks = std::min<int64_t>((words + pp.piece_words - 1) / pp.piece_words, 8 * (int64_t)sm_count());
         prep_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), tb, 0, cs>>>(pp);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "input pre-pass launch");

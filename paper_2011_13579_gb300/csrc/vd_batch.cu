@@ -41,15 +41,18 @@ using vd::PrepJob;
 
 // One block per packet: expand its transmitted values to beta int8 LLRs per
 // stage, 0 at erased positions (vd_prep.cuh).
-__global__ void prep_batch_kernel(const PrepBatchParams p) {
+__global__ void __launch_bounds__(128) prep_batch_kernel(const __grid_constant__ PrepBatchParams p) {
     const int64_t j = blockIdx.x;
     if (j >= p.n_jobs) return;
     const PrepJob jb = p.jobs[j];
     const PrepCode &c = p.codes[jb.code_slot];
-    // the packet's last kept value bounds every read (steps past T read nothing)
-    const int64_t kept_end = jb.src_off + (jb.T / c.period) * c.kept_per_period + c.kept_prefix[jb.T % c.period];
-    vd::prep_expand(jb.src ? jb.src : p.src, jb.src_off, kept_end, jb.llr_type, jb.T, c.beta, c.period,
-                    c.kept_per_period, c.punct, p.dst + jb.dst_off, threadIdx.x, blockDim.x);
+    // the packet's last kept value bounds every read; a packet of many bytes goes in pieces
+    const int64_t bytes = jb.T * c.beta, piece = vd::prep_piece_words(c.table, 1 << 20);
+    const int64_t kept = piece / c.table.words * c.table.kept;
+    for (int64_t at = 0, k = 0; 4 * at < bytes; at += piece, k += kept)
+        vd::prep_piece(jb.src ? jb.src : p.src, jb.src_off + k, jb.src_off + jb.n_kept, jb.llr_type,
+                       (uint32_t)(bytes - 4 * at < 4 * piece ? bytes - 4 * at : 4 * piece), c.table,
+                       p.dst + jb.dst_off + 4 * at, threadIdx.x, blockDim.x);
 }
 
 // ----------------------------------------------------------------- tuner
@@ -343,12 +346,7 @@ extern "C" vd_status vd_batch_plan_create(vd_batch_plan **out, const vd_code *co
     int64_t int_bytes = 0;
     memset(&pl->prep, 0, sizeof pl->prep);
     for (int i = 0; i < n_codes; ++i) {
-        PrepCode &pc = pl->prep.codes[i];
-        pc.beta = codes[i]->beta;
-        pc.period = codes[i]->period;
-        pc.kept_per_period = codes[i]->kept_per_period;
-        memcpy(pc.punct, codes[i]->punct, sizeof pc.punct);
-        memcpy(pc.kept_prefix, codes[i]->kept_prefix, sizeof pc.kept_prefix);
+        vd::fill_prep_code(codes[i], &pl->prep.codes[i]);
     }
     for (int64_t i = 0; i < n_packets; ++i) {
         const vd_packet &p = packets[i];
@@ -360,6 +358,7 @@ extern "C" vd_status vd_batch_plan_create(vd_batch_plan **out, const vd_code *co
             j.src_off = p.llr_offset;
             j.dst_off = int_bytes;
             j.T = T;
+            j.n_kept = vd_num_kept(c, T);
             j.code_slot = p.code_id;
             j.llr_type = p.llr_type;
             jobs.push_back(j);
@@ -671,10 +670,7 @@ cudaError_t launch_prep_batch(const PrepBatchParams &p, cudaStream_t st) {
 
 void fill_prep_code(const vd_code *c, PrepCode *pc) {
     pc->beta = c->beta;
-    pc->period = c->period;
-    pc->kept_per_period = c->kept_per_period;
-    memcpy(pc->punct, c->punct, sizeof pc->punct);
-    memcpy(pc->kept_prefix, c->kept_prefix, sizeof pc->kept_prefix);
+    pc->table = prep_table(c->beta, c->period, c->punct);
 }
 
 }  // namespace vd

@@ -5,6 +5,7 @@
 
 #include "../../include/vd.h"
 #include "vd_launch.h"
+#include "vd_prep.cuh"
 
 struct vd_code {
     int K, beta;
@@ -39,16 +40,15 @@ namespace vd {
 constexpr int kMaxBatchCodes = 16;
 
 struct PrepCode {
-    int beta, period, kept_per_period, pad;
-    uint8_t punct[4][8];
-    int kept_prefix[9];
+    int beta;
+    PrepTable table;
 };
 
 struct PrepJob {
     const uint8_t *src;  // NULL: the launch's source arena; else the packet's own values (device)
     int64_t src_off;     // first kept value of the packet in the source (values)
     int64_t dst_off;     // byte offset of the packet's [T][beta] int8 in the destination
-    int64_t T;
+    int64_t T, n_kept;   // stages, kept values
     int32_t code_slot;
     int32_t llr_type;
 };

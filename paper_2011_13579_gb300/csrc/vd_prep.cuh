@@ -1,12 +1,15 @@
 // Input pre-pass helper: expands transmitted (kept) LLR values to beta int8
 // LLRs per stage, inserting 0 at the positions a puncturing pattern erases,
-// sign-extending 4-bit values and mapping hard decisions to +-1.  The kept values are stage-major with b
-// ascending, so the values of puncturing period g (stages g*period ..) start
-// at g * kept_per_period.
+// sign-extending 4-bit values and mapping hard decisions to +-1.  The kept
+// values are stage-major with b ascending.
 //
-// A thread produces m whole periods at a time, m chosen so that their
-// m * period * beta output bytes are a whole number of 32-bit words: the
-// stores of a warp then cover full, contiguous sectors.
+// What bounds it: memory, once a thread's work is small.  The pattern of erased
+// positions repeats over a cycle of output words (the least common multiple of a
+// puncturing period's bytes and 4), so each output word is four kept values in
+// a row, read as one unaligned field, and a byte permute that puts them, or zero,
+// in their places: a table gives both per word of the cycle.  A warp writes 128
+// contiguous bytes at a time.  Measured (GB300, us, against a thread per puncturing period with byte
+// loads): 43,690 punctured packets (175 MB in, 216 MB out) 245 -> 107; 3 M stages of 4-bit values 18.4 -> 7.1.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -15,124 +18,111 @@
 
 namespace vd {
 
-// One value of the kept stream (int8; 4-bit two per byte, low nibble
-// first; or a hard decision, eight per byte, bit 0 first, mapped to +1 for
-// bit 0 and -1 for bit 1); 0 at or past n_kept (the end of this packet's
-// values), which is never read.
-__device__ __forceinline__ int8_t prep_kept_value(const uint8_t *src, int64_t k, int64_t n_kept, int llr_type) {
-    if (k >= n_kept) return 0;
-    if (llr_type == VD_LLR_HARD) return ((src[k >> 3] >> (k & 7)) & 1u) ? (int8_t)-1 : (int8_t)1;
-    if (llr_type == VD_LLR_S4) {
-        const uint8_t byte = src[k >> 1];
-        const uint8_t nib = (k & 1) ? (byte >> 4) : (byte & 0x0F);
-        return (int8_t)((int8_t)(nib << 4) >> 4);
-    }
-    return (int8_t)src[k];
-}
+constexpr int kPrepWords = 24;   // words of a cycle: at most 21 (period 7 of 3 outputs, 5 or 7 of 4 bytes a period less)
 
-// The same for a compile-time (period, beta): the loops unroll, so a step's
-// loads are independent and issue together.
-template <int P, int B>
-__device__ __forceinline__ void prep_expand_fixed(const uint8_t *src, int64_t k0, int64_t n_kept, int llr_type,
-                                                  int64_t T, int kept_per_period, const uint8_t (&punct)[4][8],
-                                                  int8_t *dst, int64_t tid, int64_t nthr) {
-    constexpr int GB = P * B;
-    constexpr int M = (GB % 4 == 0) ? 1 : (GB % 2 == 0) ? 2 : 4;
-    constexpr int SPAN = M * GB;
-    static_assert(SPAN <= 16, "step too wide");
-    bool keep[B][P];
-#pragma unroll
-    for (int b = 0; b < B; ++b)
-#pragma unroll
-        for (int ph = 0; ph < P; ++ph) keep[b][ph] = punct[b][ph] != 0;
-    const int64_t n_groups = (T + P - 1) / P;
-    const int64_t n_steps = (n_groups + M - 1) / M;
-    const int64_t full_steps = (T * B) / SPAN;   // steps wholly inside the output
-    for (int64_t st = tid; st < n_steps; st += nthr) {
-        int64_t k = k0 + st * M * kept_per_period;
-        uint8_t v[SPAN];
-#pragma unroll
-        for (int i = 0; i < M; ++i)
-#pragma unroll
-            for (int ph = 0; ph < P; ++ph)
-#pragma unroll
-                for (int b = 0; b < B; ++b)
-                    v[(i * P + ph) * B + b] = keep[b][ph] ? (uint8_t)prep_kept_value(src, k++, n_kept, llr_type) : 0;
-        if (st < full_steps) {
-            uint32_t *d = reinterpret_cast<uint32_t *>(dst + st * SPAN);
-#pragma unroll
-            for (int w = 0; w < SPAN / 4; ++w)
-                d[w] = (uint32_t)v[4 * w] | ((uint32_t)v[4 * w + 1] << 8) | ((uint32_t)v[4 * w + 2] << 16) |
-                       ((uint32_t)v[4 * w + 3] << 24);
-        } else {
-#pragma unroll
-            for (int j = 0; j < SPAN; ++j)
-                if (st * SPAN + j < T * B) dst[st * SPAN + j] = (int8_t)v[j];
+// The cycle of one code: `words` output words hold `kept` kept values; word w
+// begins with the cycle's kept value first[w] (or a later one) and is the byte
+// permute sel[w] of that value and the three after it (nibble 4: zero).
+struct PrepTable {
+    int32_t words, kept;
+    uint8_t first[kPrepWords];
+    uint16_t sel[kPrepWords];
+};
+
+inline PrepTable prep_table(int beta, int period, const uint8_t (&punct)[4][8]) {
+    PrepTable t = {};
+    const int bytes = beta * period;
+    int cycle = bytes;
+    while (cycle % 4) cycle += bytes;
+    t.words = cycle / 4;
+    int k = 0;
+    for (int w = 0; w < t.words; ++w) {
+        t.first[w] = (uint8_t)k;
+        for (int i = 0; i < 4; ++i) {
+            const int j = (4 * w + i) % bytes;
+            const bool on = punct[j % beta][j / beta] != 0;
+            t.sel[w] |= (uint16_t)((on ? k - t.first[w] : 4) << (4 * i));
+            if (on) ++k;
         }
     }
+    t.kept = k;
+    return t;
 }
 
-// Expands stages [0, T) into dst ([T][beta] int8, 4-byte aligned) from the
-// kept values src[k0 .. n_kept).  Threads tid, tid + nthr, .. of the caller
-// share the work.
-__device__ __forceinline__ void prep_expand(const uint8_t *src, int64_t k0, int64_t n_kept, int llr_type,
-                                            int64_t T, int beta, int period, int kept_per_period,
-                                            const uint8_t (&punct)[4][8], int8_t *dst, int64_t tid,
-                                            int64_t nthr) {
-    // the shapes of the supported codes, unrolled
-    if (period == 2 && beta == 2)
-        return prep_expand_fixed<2, 2>(src, k0, n_kept, llr_type, T, kept_per_period, punct, dst, tid, nthr);
-    if (period == 3 && beta == 2)
-        return prep_expand_fixed<3, 2>(src, k0, n_kept, llr_type, T, kept_per_period, punct, dst, tid, nthr);
-    if (period == 1 && beta == 2)
-        return prep_expand_fixed<1, 2>(src, k0, n_kept, llr_type, T, kept_per_period, punct, dst, tid, nthr);
-    if (period == 1 && beta == 3)
-        return prep_expand_fixed<1, 3>(src, k0, n_kept, llr_type, T, kept_per_period, punct, dst, tid, nthr);
-    const int gb = period * beta;                               // output bytes per period
-    const int m = (gb % 4 == 0) ? 1 : (gb % 2 == 0) ? 2 : 4;   // periods per thread step
-    const int span = m * gb;                                    // bytes per thread step
-    const int64_t out_bytes = T * beta;
-    const int64_t n_groups = (T + period - 1) / period;
-    const int64_t n_steps = (n_groups + m - 1) / m;
-    for (int64_t st = tid; st < n_steps; st += nthr) {
-        const int64_t byte0 = st * span;
-        const int64_t g0 = st * m;
-        if (span <= 16 && byte0 + span <= out_bytes) {
-            // whole step inside the output: assemble up to 16 bytes in two
-            // 64-bit registers, store them as 32-bit words
-            uint64_t lo = 0, hi = 0;
-            int pos = 0;
-            for (int i = 0; i < m; ++i) {
-                int64_t k = k0 + (g0 + i) * kept_per_period;
-                for (int ph = 0; ph < period; ++ph) {
-                    for (int b = 0; b < beta; ++b, ++pos) {
-                        const int8_t x = punct[b][ph] ? prep_kept_value(src, k++, n_kept, llr_type) : (int8_t)0;
-                        const uint64_t v = (uint64_t)(uint8_t)x;
-                        if (pos < 8) lo |= v << (8 * pos);
-                        else hi |= v << (8 * (pos - 8));
-                    }
-                }
+// Expands output words [0, n) of a piece that begins a cycle: out_bytes bytes at dst (4-byte aligned)
+// from the kept values k0 .. kept_end of src.  Threads tid, tid + nthr, .. of the
+// caller share the work.  A piece is short enough for 32-bit offsets, which is most of
+// what a word costs: an earlier form with 64-bit ones took 85 instructions a word.
+// Only aligned 32-bit words that hold part of a kept value before kept_end are read.
+template <int BITS>
+__device__ __forceinline__ void prep_piece(const uint8_t *src, int64_t k0, int64_t kept_end, uint32_t out_bytes,
+                                           const PrepTable &t, int8_t *dst, uint32_t tid, uint32_t nthr) {
+    const uint64_t bit0 = (uint64_t)k0 * BITS;
+    const uint8_t *a = src + (bit0 >> 3);
+    const uint32_t mis = (uint32_t)(reinterpret_cast<uintptr_t>(a) & 3u);
+    const uint32_t *in = reinterpret_cast<const uint32_t *>(a - mis);
+    const uint32_t b0 = 8u * mis + (uint32_t)(bit0 & 7u);                  // first kept value, in bits from `in`
+    const uint64_t left = (uint64_t)(kept_end - k0) * BITS + b0;
+    const uint32_t n_in = left > 0x7FFFFFE0ull ? 0x3FFFFFFu : (uint32_t)((left + 31u) >> 5);   // words that may be read
+    const uint32_t n_full = out_bytes / 4, n_words = (out_bytes + 3) / 4;
+    const uint32_t words = (uint32_t)t.words, kept = (uint32_t)t.kept;
+    const uint32_t c0 = tid / words, dc = nthr / words, dw = nthr - dc * words, dk = dc * kept;
+    uint32_t w = tid - c0 * words, k = c0 * kept;
+    uint32_t *out = reinterpret_cast<uint32_t *>(dst);
+    constexpr int N = 4;             // words in flight
+    for (uint32_t i0 = tid; i0 < n_words; i0 += N * nthr) {
+        uint32_t lo[N], hi[N], sh[N], sel[N];
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            const uint32_t bit = b0 + (k + t.first[w]) * BITS;
+            const uint32_t j = bit >> 5;
+            sh[n] = bit & 31u;
+            sel[n] = t.sel[w];
+            // a word past the last one reads nothing that is used
+            lo[n] = j < n_in ? __ldg(in + j) : 0u;
+            hi[n] = j + 1u < n_in && sh[n] + 4u * BITS > 32u ? __ldg(in + j + 1) : 0u;
+            k += dk;
+            w += dw;
+            if (w >= words) {
+                w -= words;
+                k += kept;
             }
-            uint32_t *d = reinterpret_cast<uint32_t *>(dst + byte0);
-            d[0] = (uint32_t)lo;
-            if (span > 4) d[1] = (uint32_t)(lo >> 32);
-            if (span > 8) d[2] = (uint32_t)hi;
-            if (span > 12) d[3] = (uint32_t)(hi >> 32);
-        } else {
-            // the last, partial step (or an unusually long period): byte stores
-            for (int i = 0; i < m; ++i) {
-                const int64_t g = g0 + i;
-                int64_t k = k0 + g * kept_per_period;
-                for (int ph = 0; ph < period; ++ph) {
-                    const int64_t t = g * period + ph;
-                    for (int b = 0; b < beta; ++b) {
-                        const int8_t x = punct[b][ph] ? prep_kept_value(src, k++, n_kept, llr_type) : (int8_t)0;
-                        if (t < T) dst[t * beta + b] = x;
-                    }
-                }
+        }
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            const uint32_t i = i0 + n * nthr;
+            uint32_t x = __funnelshift_r(lo[n], hi[n], sh[n]);
+            if constexpr (BITS == 4) {
+                x &= 0xFFFFu;
+                x = (x | (x << 8)) & 0x00FF00FFu;
+                x = (x | (x << 4)) & 0x0F0F0F0Fu;
+                x |= (x & 0x08080808u) * 0x1Eu;                             // sign: 0x08 -> 0xF8
+            } else if constexpr (BITS == 1) {
+                // bit 0 -> 1, bit 1 -> -1
+                x = 0x01010101u + (((x & 0xFu) * 0x00204081u) & 0x01010101u) * 0xFEu;
+            }
+            uint32_t y;
+            asm("prmt.b32 %0, %1, %2, %3;" : "=r"(y) : "r"(x), "r"(0u), "r"(sel[n]));
+            if (i < n_full) {
+                out[i] = y;
+            } else if (i < n_words) {
+                for (uint32_t b = 0; 4 * i + b < out_bytes; ++b) dst[4 * i + b] = (int8_t)(y >> (8 * b));
             }
         }
     }
+}
+
+__device__ __forceinline__ void prep_piece(const uint8_t *src, int64_t k0, int64_t kept_end, int llr_type,
+                                           uint32_t out_bytes, const PrepTable &t, int8_t *dst, uint32_t tid,
+                                           uint32_t nthr) {
+    if (llr_type == VD_LLR_HARD) prep_piece<1>(src, k0, kept_end, out_bytes, t, dst, tid, nthr);
+    else if (llr_type == VD_LLR_S4) prep_piece<4>(src, k0, kept_end, out_bytes, t, dst, tid, nthr);
+    else prep_piece<8>(src, k0, kept_end, out_bytes, t, dst, tid, nthr);
+}
+
+// Output words of a piece of about `target` words: whole cycles.
+__host__ __device__ inline int64_t prep_piece_words(const PrepTable &t, int64_t target) {
+    return (target + t.words - 1) / t.words * t.words;
 }
 
 }  // namespace vd

@@ -238,6 +238,7 @@ bool launch_batch(vd_server *s, Slot &sl) {
                                                  : (int64_t)r->in_off;
         j.dst_off = (int64_t)r->prep_off;
         j.T = r->T;
+        j.n_kept = vd_num_kept(s->codes[(size_t)r->code_id], r->T);
         j.code_slot = r->code_id;
         j.llr_type = r->llr_type;
     }
