@@ -12,13 +12,16 @@
 // et al., SC 2011) with key (seed, stream_id) on counter block k / 4, turned
 // into four normals by the Box-Muller transform in double precision.
 //
-// What bounds it: the 64-bit integer products of Philox.  In double precision
-// alone the transform bound it instead (the fp64 units give two lanes per clock and SM): 732 us for
+// What bounds it: instruction issue (74% of the cycles; 174 instructions a value,
+// the 64-bit integer products of Philox first).  In double precision
+// alone the transform bound it (the fp64 units give two lanes per clock and SM): 732 us for
 // 8.4 M int8 values, on GB300.  The transform is therefore taken in single precision with an
 // error bound, which settles the quantised value unless a rounding border
-// lies within the bound; a thread with such a value (2 in 10^4 for int8, 1 in 100 for half
-// precision) takes its eight values from the double-precision transform instead.  The bytes are those of
-// the double-precision transform.  Measured: 8.4 M int8 values (2^22 bits, K=7) 732 -> 76 us.
+// lies within the bound; a pair with such a value (1 in 10^4 for int8, 1 in 300 for half
+// precision) comes from the double-precision transform instead.  The bytes are those of
+// the double-precision transform.  Measured, 8.4 M int8 values (2^22 bits, K=7): 732 us; with logf,
+// log1pf and sincospif and eight values at a time in double precision 77; with the
+// polynomials below and two at a time 56.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -91,19 +94,6 @@ __device__ __forceinline__ uint32_t info_window(const TxParams &p, int64_t lo) {
     return v;
 }
 
-// Eight normals of blocks 2 j and 2 j + 1, in double precision.
-__device__ __forceinline__ void normals(uint64_t (&w)[2][4], double (&z)[8]) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const double u = unit53(w[h][2 * q]), v = unit53(w[h][2 * q + 1]);
-            const double rad = sqrt(-2.0 * log(u)), ang = 2.0 * 3.14159265358979323846 * v;
-            z[4 * h + 2 * q] = rad * cos(ang);
-            z[4 * h + 2 * q + 1] = rad * sin(ang);
-        }
-}
-
 // The quantised value of a sample as the bits it has in the output.
 template <int TYPE>
 __device__ __forceinline__ uint32_t quantise(double y, double inv_var2) {
@@ -113,110 +103,141 @@ __device__ __forceinline__ uint32_t quantise(double y, double inv_var2) {
     else return y < 0.0 ? 1u : 0u;
 }
 
-// Double precision for a thread whose values single precision leaves open:
-// eight 16-bit fields.
+// Double precision for a pair of values that single precision leaves open (two 16-bit fields).
 template <int TYPE>
-__device__ __noinline__ uint4 exact_values(uint64_t j, uint64_t seed, uint64_t stream_id, uint32_t cbits, double sigma,
-                                           double inv_var2) {
-    uint64_t w[2][4] = {{2 * j, 0ull, 0ull, 0ull}, {2 * j + 1, 0ull, 0ull, 0ull}};
-    philox4x64(w[0], seed, stream_id);
-    philox4x64(w[1], seed, stream_id);
-    double z[8];
-    normals(w, z);
-    uint32_t q[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const double y = (((cbits >> i) & 1u) ? -1.0 : 1.0) + sigma * z[i];
-        q[i] = quantise<TYPE>(y, inv_var2);
-    }
-    return make_uint4(q[0] | q[1] << 16, q[2] | q[3] << 16, q[4] | q[5] << 16, q[6] | q[7] << 16);
+__device__ __noinline__ uint32_t exact_pair(uint64_t wu, uint64_t wv, uint32_t cbits, double sigma, double inv_var2) {
+    const double u = unit53(wu), v = unit53(wv);
+    const double rad = sqrt(-2.0 * log(u)), ang = 2.0 * 3.14159265358979323846 * v;
+    const double y0 = ((cbits & 1u) ? -1.0 : 1.0) + sigma * (rad * cos(ang));
+    const double y1 = ((cbits & 2u) ? -1.0 : 1.0) + sigma * (rad * sin(ang));
+    return quantise<TYPE>(y0, inv_var2) | quantise<TYPE>(y1, inv_var2) << 16;
 }
 
-// A Box-Muller pair in single precision.  u = U 2^-53 and v = V 2^-53 enter as
-// integers, so that 1 - u and the angle's offset from the nearest quarter
-// turn are exact before they are rounded to 24 bits.  Errors, with logf,
-// log1pf, sinpif and cospif good to 2 ulp and sqrtf to half of one: ln u
-// 4e-7 of itself (6e-8 of u or 1 - u, at most 1.45 times that in the logarithm, and 2 ulp), rad half of that and
-// 6e-8; the sine and cosine 5e-8 (the angle) and 2.4e-7.  So cos and sin
-// times rad are off by less than 6e-7 rad.
+// ln(U 2^-53) for U in 1 .. 2^53.  U 2^-53 = (1 + f) 2^e with 1 + f in [2/3, 4/3), f
+// from an exact integer difference; ln(1 + f) = f q(f), q the polynomial of degree 10
+// that interpolates ln(1 + f) / f at the Chebyshev nodes of [-1/3, 1/3].  Within 1.7e-7 of
+// itself (checked against 64 bits over all binades and both ends).
+__device__ __forceinline__ float ln_u53(uint64_t U) {
+    const int lz = __clzll((long long)U);
+    const uint64_t M = U << (lz - 10);                       // in [2^53, 2^54)
+    const bool up = M >= (1ull << 55) / 3ull;                // 1 + f = M 2^-54, else M 2^-53
+    const float f = __ll2float_rn((long long)(M - (up ? 1ull << 54 : 1ull << 53))) * (up ? 0x1.0p-54f : 0x1.0p-53f);
+    float q = 0.11900901794433594f;
+    q = fmaf(q, f, -0.13038060069084167f);
+    q = fmaf(q, f, 0.10781308263540268f);
+    q = fmaf(q, f, -0.12143635004758835f);
+    q = fmaf(q, f, 0.14302155375480652f);
+    q = fmaf(q, f, -0.16684426367282867f);
+    q = fmaf(q, f, 0.1999966949224472f);
+    q = fmaf(q, f, -0.24999643862247467f);
+    q = fmaf(q, f, 0.3333333432674408f);
+    q = fmaf(q, f, -0.5f);
+    q = fmaf(q, f, 1.0f);
+    return fmaf((float)(10 - lz + (up ? 1 : 0)), 0.693147180559945f, f * q);
+}
+
+// A Box-Muller pair in single precision; u = U 2^-53 and v = V 2^-53 enter as
+// integers, so that the angle's offset from the nearest quarter turn is exact before it is rounded
+// to 24 bits.  Errors: rad 2.1e-7 of itself (half of the logarithm's 1.7e-7, 2^-23 of the
+// square root), the cosine and sine (Taylor polynomials on an eighth of a
+// turn) 8.7e-8 and 4.7e-8 for the angle: rad times either is off by less than 3.5e-7 rad.
 __device__ __forceinline__ void pair_f32(uint64_t wu, uint64_t wv, float &rad, float &c, float &s) {
-    const uint64_t U = (wu >> 11) + 1ull, V = (wv >> 11) + 1ull;
-    const bool low = U <= (1ull << 52);
-    const float a = __ull2float_rn(low ? U : (1ull << 53) - U) * 0x1.0p-53f;
-    const float ln = low ? logf(a) : log1pf(-a);
-    rad = sqrtf(-2.0f * ln);
+    const float x = -2.0f * ln_u53((wu >> 11) + 1ull);
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(rad) : "f"(x));
+    const uint64_t V = (wv >> 11) + 1ull;
     const uint64_t quad = (V + (1ull << 50)) >> 51;
     const float r = __ll2float_rn((long long)(V - (quad << 51))) * 0x1.0p-52f;   // half turns, at most 1/4
-    float sn, cs;
-    sincospif(r, &sn, &cs);
+    const float t = r * r;
+    float sn = 0.0821458866f;                      // pi^9 / 9!
+    sn = fmaf(sn, t, -0.599264529f);
+    sn = fmaf(sn, t, 2.55016404f);
+    sn = fmaf(sn, t, -5.16771278f);
+    sn = fmaf(sn, t, 3.14159265f);
+    sn *= r;
+    float cs = -0.0258068913f;                     // -pi^10 / 10!
+    cs = fmaf(cs, t, 0.235330630f);
+    cs = fmaf(cs, t, -1.33526277f);
+    cs = fmaf(cs, t, 4.05871213f);
+    cs = fmaf(cs, t, -4.93480220f);
+    cs = fmaf(cs, t, 1.0f);
     const bool odd = quad & 1ull;
-    const float x = odd ? sn : cs, y = odd ? cs : sn;
-    c = (quad + 1ull) & 2ull ? -x : x;   // quarter turns 1, 2: negative cosine
-    s = quad & 2ull ? -y : y;            // quarter turns 2, 3: negative sine
+    const float p = odd ? sn : cs, q = odd ? cs : sn;
+    c = (quad + 1ull) & 2ull ? -p : p;   // quarter turns 1, 2: negative cosine
+    s = quad & 2ull ? -q : q;            // quarter turns 2, 3: negative sine
 }
 
 template <int TYPE>
-__global__ void __launch_bounds__(256) transmit_kernel(const TxParams p) {
+__global__ void __launch_bounds__(256) transmit_kernel(const __grid_constant__ TxParams p) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t k0 = 8 * j;
     if (k0 >= p.n_kept) return;
     // encoder outputs of the thread's kept values: at most eight stages, one window of input bits
     int64_t g = p.kept_per_period == 1 ? k0 : (int64_t)__umul64hi((uint64_t)k0, p.kpp_magic);
     int r = (int)(k0 - g * p.kept_per_period);
-    int64_t tg = g * p.period;                        // first stage of the period
-    const int64_t t0 = tg + p.pos_phase[r];
+    const int64_t t0 = g * p.period + p.pos_phase[r];
     const uint32_t win = info_window(p, t0 - (p.K - 1));
+    // output b of all stages of the window at once: bit dt of o[b] is stage t0 + dt
+    uint32_t o[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        if (b < p.beta) {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) o[b] ^= (p.gens[b] >> i & 1u) ? win >> i : 0u;
+        }
+    }
     uint32_t cbits = 0;
+    int dt = 0 - p.pos_phase[r];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        const int dt = (int)(tg - t0) + p.pos_phase[r];
-        const uint32_t reg = (win >> dt) & ((1u << p.K) - 1u);
-        cbits |= ((uint32_t)__popc(p.gens[p.pos_b[r]] & reg) & 1u) << i;
+        const int b = p.pos_b[r];
+        const uint32_t x = b == 0 ? o[0] : b == 1 ? o[1] : b == 2 ? o[2] : o[3];
+        cbits |= ((x >> (dt + p.pos_phase[r])) & 1u) << i;
         if (++r == p.kept_per_period) {
             r = 0;
-            tg += p.period;
+            dt += p.period;
         }
     }
     uint64_t w[2][4] = {{(uint64_t)(2 * j), 0ull, 0ull, 0ull}, {(uint64_t)(2 * j + 1), 0ull, 0ull, 0ull}};
     philox4x64(w[0], p.seed, p.stream_id);
     philox4x64(w[1], p.seed, p.stream_id);
     uint32_t q[8];
-    bool open = false;
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
+        const uint64_t wu = w[m >> 1][2 * (m & 1)], wv = w[m >> 1][2 * (m & 1) + 1];
         float rad, cs[2];
-        pair_f32(w[m >> 1][2 * (m & 1)], w[m >> 1][2 * (m & 1) + 1], rad, cs[0], cs[1]);
-        // y = +-1 + sigma z: the pair's error, the rounding of sigma, of the
-        // product and of the sum (2.4e-7 together), each with room to spare
-        const float srad = p.sigma_f * rad, ey = 1.2e-6f * srad + 3e-7f;
+        pair_f32(wu, wv, rad, cs[0], cs[1]);
+        // y = +-1 + sigma z: the pair's 3.5e-7 sigma rad, the roundings of sigma, of
+        // sigma rad and of the sum (6e-8 each of theirs), with half as much again to spare
+        const float srad = p.sigma_f * rad, ey = 8e-7f * srad + 1.5e-7f;
+        bool open = false;
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const int i = 2 * m + k;
             const float y = fmaf(srad, cs[k], ((cbits >> i) & 1u) ? -1.0f : 1.0f);
-            uint32_t lo, hi;
-            if constexpr (TYPE == VD_LLR_S8) {
-                lo = (uint32_t)(int)fminf(fmaxf(rintf(32.0f * (y - ey)), -127.0f), 127.0f) & 0xFFu;
-                hi = (uint32_t)(int)fminf(fmaxf(rintf(32.0f * (y + ey)), -127.0f), 127.0f) & 0xFFu;
-            } else if constexpr (TYPE == VD_LLR_S4) {
-                lo = (uint32_t)(int)fminf(fmaxf(rintf(2.0f * (y - ey)), -7.0f), 7.0f) & 0xFu;
-                hi = (uint32_t)(int)fminf(fmaxf(rintf(2.0f * (y + ey)), -7.0f), 7.0f) & 0xFu;
+            if constexpr (TYPE == VD_LLR_S8 || TYPE == VD_LLR_S4) {
+                // scaled by a power of two and clipped; adding 1.5 2^23 rounds to the nearest
+                // integer, ties to even, and leaves it in the low bits.  Open: within the bound of
+                // a half-integer, unless well past the clip.
+                constexpr float SCALE = TYPE == VD_LLR_S8 ? 32.0f : 2.0f, TOP = TYPE == VD_LLR_S8 ? 127.0f : 7.0f;
+                const float t = SCALE * y, et = SCALE * ey;
+                const float tc = fminf(fmaxf(t, -TOP), TOP);
+                const float big = tc + 12582912.0f;
+                q[i] = __float_as_uint(big) & (TYPE == VD_LLR_S8 ? 0xFFu : 0xFu);
+                open |= fabsf(tc - (big - 12582912.0f)) > 0.5f - et && fabsf(t) < TOP + 1.0f + et;
             } else if constexpr (TYPE == VD_LLR_F16) {
                 const float x = y * p.inv_var2_f, ex = ey * p.inv_var2_f + 3e-7f * fabsf(x);
-                lo = __half_as_ushort(__float2half_rn(x - ex));
-                hi = __half_as_ushort(__float2half_rn(x + ex));
+                q[i] = __half_as_ushort(__float2half_rn(x - ex));
+                open |= q[i] != (uint32_t)__half_as_ushort(__float2half_rn(x + ex));
             } else {
-                lo = y - ey < 0.0f ? 1u : 0u;
-                hi = y + ey < 0.0f ? 1u : 0u;
+                q[i] = y < 0.0f ? 1u : 0u;
+                open |= fabsf(y) <= ey;
             }
-            q[i] = lo;
-            open |= lo != hi;
         }
-    }
-    if (open) {
-        const uint4 x = exact_values<TYPE>((uint64_t)j, p.seed, p.stream_id, cbits, p.sigma, p.inv_var2);
-        const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int i = 0; i < 8; ++i) q[i] = (xs[i >> 1] >> (16 * (i & 1))) & 0xFFFFu;
+        if (open) {
+            const uint32_t e = exact_pair<TYPE>(wu, wv, cbits >> (2 * m), p.sigma, p.inv_var2);
+            q[2 * m] = e & 0xFFFFu;
+            q[2 * m + 1] = e >> 16;
+        }
     }
     const int n = p.n_kept - k0 < 8 ? (int)(p.n_kept - k0) : 8;   // values of this thread
     if constexpr (TYPE == VD_LLR_S8) {
