@@ -926,10 +926,13 @@ __device__ __forceinline__ bool forward_pair(const FrameTask (&ft)[2], uint32_t 
             hook(Sc, c);
         });
     };
-    // the lanes that run together take the copy with the test if one of them needs it
+    // The condition is the same for all lanes of a group, and so is the copy that they take: both
+    // copies shuffle over gmask, which is defined only if the group's lanes run the same one.
+    // (Groups of a warp may differ; no vote over them, since no set of lanes is known to be
+    // together here: their chunk counts differ.)
     const int rc0 = reset_at0 >= 0 ? reset_at0 / U : -1, rc1 = reset_at1 >= 0 ? reset_at1 / U : -1;
     for (int c = 0; c < nchunks; ++c) {
-        if (HEADSTART_COPY && __any_sync(__activemask(), c == rc0 || c == rc1)) chunk(std::true_type{}, c);
+        if (HEADSTART_COPY && (c == rc0 || c == rc1)) chunk(std::true_type{}, c);
         else chunk(std::false_type{}, c);
     }
 
