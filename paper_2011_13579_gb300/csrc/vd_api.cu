@@ -321,25 +321,35 @@ struct Plan {
     size_t smem;               // SPLIT, WIDE
 };
 
+// SMs of the current device; 0 (and nothing kept) if the query fails.
 int sm_count() {
     static std::mutex mu;
     static std::map<int, int> cache;
-    int dev = 0;
-    cudaGetDevice(&dev);
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
     std::lock_guard<std::mutex> lk(mu);
     auto it = cache.find(dev);
     if (it != cache.end()) return it->second;
-    int n = 0;
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
     return cache[dev] = n;
 }
 
-// Resident blocks per SM of the persistent or the one-wave stream kernel, per device and shape.
+// Resident blocks per SM of the persistent or the one-wave stream kernel, per
+// device and shape; 0 (and nothing kept) if the query fails.
 int blocks_per_sm(bool persistent, int K, int lanes, bool r4) {
     static std::mutex mu;
     static std::map<std::tuple<int, bool, int, int, bool>, int> cache;
     int dev = 0;
-    cudaGetDevice(&dev);
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
     std::lock_guard<std::mutex> lk(mu);
     const auto key = std::make_tuple(dev, persistent, K, lanes, r4);
     auto it = cache.find(key);
@@ -348,10 +358,9 @@ int blocks_per_sm(bool persistent, int K, int lanes, bool r4) {
     if ((persistent ? vd::stream_persistent_occupancy(K, lanes, r4, &bps)
                     : vd::stream_wave_occupancy(K, lanes, r4, &bps)) != cudaSuccess) {
         cudaGetLastError();
-        bps = 0;
+        return 0;
     }
-    cache[key] = bps;
-    return bps;
+    return cache[key] = bps;
 }
 
 // The wide form, while its blocks make at most this many waves of what the SMs
@@ -381,12 +390,15 @@ size_t wave_scratch(int64_t n_pairs, int lanes, int64_t wmax, const vd::KernelGe
 // while they are (8.4 M: 314 against 362), then eight again (10 M 437 / 532,
 // 16.8 M 590 / 621, 20 M 739 / 801 against the persistent form with four) while
 // the survivors of all pairs take no more memory than the persistent form's.
+// The persistent form is sized by its resident blocks: where their number is not
+// known, or zero, the one-wave form runs.
 void choose_shape(const vd_code *c, bool r4, int64_t n_pairs, int64_t wmax, int *lanes, Form *form) {
     const int64_t n_sm = sm_count();
     auto resident_pairs = [&](int l) { return n_sm * blocks_per_sm(false, c->K, l, r4) * (vd::kThreads / l); };
     if (c->kind == vd::KIND_K7_R2) {
         *lanes = n_pairs <= resident_pairs(2) ? 2 : 1;
-        *form = *lanes == 2 || (n_pairs + 31) / 32 <= 2 * 4 * n_sm ? Form::WAVE : Form::PERSISTENT;
+        const bool fits = *lanes == 2 || (n_pairs + 31) / 32 <= 2 * 4 * n_sm;
+        *form = fits || n_sm * blocks_per_sm(true, c->K, *lanes, r4) < 1 ? Form::WAVE : Form::PERSISTENT;
         return;
     }
     *form = Form::WAVE;
@@ -401,7 +413,7 @@ void choose_shape(const vd_code *c, bool r4, int64_t n_pairs, int64_t wmax, int 
     if (!geometry(c->kind, 8, r4, &g8) || !geometry(c->kind, 4, r4, &g4)) return;
     const size_t persistent = 2u * (size_t)(n_sm * blocks_per_sm(true, c->K, 4, r4)) * vd::kThreads *
                               (size_t)((wmax + g4.U - 1) / g4.U * g4.U) * g4.NW * 4u;
-    if (wave_scratch(n_pairs, 8, wmax, g8, &blocks) > persistent) {
+    if (persistent > 0 && wave_scratch(n_pairs, 8, wmax, g8, &blocks) > persistent) {
         *lanes = 4;
         *form = Form::PERSISTENT;
     }
