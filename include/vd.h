@@ -175,14 +175,36 @@ vd_status vd_decode_host(const vd_code *code, int n_streams, const void *const *
                          void *stream);
 
 /*
- * The configuration vd_decode uses for this code and LLR type when its tune
- * argument is NULL: f, v and radix as given, and the lanes per frame pair and
- * threads per block it picks (for streams of many frames; few frames take the
- * other forms of vd_decode).  The decoded bits depend only on f, v and the
- * flags, so this is what a reference decoder needs to reproduce a call.
+ * A shape that vd_decode has for streams of many frames of this code and LLR
+ * type, as a vd_tune: f, v and radix as given (2 for fp16), the default lanes per frame
+ * pair and threads per block.  Passing it on names the lanes, so vd_decode takes that
+ * shape for a stream of any length; with tune NULL it goes by the stream instead
+ * (vd_decode_shape tells what runs).  The decoded bits depend only on f, v and
+ * the flags, so that is what a reference decoder needs to reproduce a call.
  * VD_EINVAL on bad arguments, VD_EUNSUPPORTED if there is no kernel.
  */
 vd_status vd_get_tune(const vd_code *code, int llr_type, int f, int v, int radix, vd_tune *out);
+
+/* Kernel forms of vd_decode (vd_shape.form; vd_tune.form names the first two). */
+enum { VD_FORM_PERSISTENT = 1, VD_FORM_ONE_WAVE = 2, VD_FORM_FEW_FRAMES = 3, VD_FORM_SEGMENTS = 4 };
+
+typedef struct vd_shape {
+    int32_t form;            /* VD_FORM_* */
+    int32_t radix;           /* of the steps that run: 2 or 4 */
+    int32_t lanes;           /* threads per pair of frames (VD_FORM_SEGMENTS: of segments) */
+    int32_t warp_pairs;      /* pairs that a warp decodes at once */
+    int64_t blocks;          /* of the launch */
+    int32_t blocks_per_sm;   /* resident at once, for VD_FORM_PERSISTENT and integer VD_FORM_ONE_WAVE; 0 otherwise */
+    int32_t cluster;         /* blocks that share a frame (VD_FORM_SEGMENTS; 1 otherwise) */
+    int32_t reserved[4];
+} vd_shape;
+
+/*
+ * What vd_decode runs for these arguments on the current device.  No launch, no
+ * allocation.  n_info > 0; other errors as vd_decode.
+ */
+vd_status vd_decode_shape(const vd_code *code, int llr_type, int64_t n_info, int f, int v, int radix, uint32_t flags,
+                          const vd_tune *tune, vd_shape *out);
 
 /* ------------------------------------------------------------------ batches
  *

@@ -25,13 +25,15 @@ __all__ = [
     "vd_batch_plan_info", "vd_batch_plan_packet_tune", "vd_batch_plan_status", "vd_batch_plan_destroy",
     "VdPacket", "VdBatchInfo", "BatchPlan", "VdServerConfig", "VdCompletion", "VdServerStats",
     "Server", "vd_server_create", "vd_server_submit", "vd_server_poll", "vd_server_stats_get",
-    "vd_server_destroy", "vd_server_replay", "vd_server_submit_device", "vd_server_submit_many", "vd_bm_gate", "vd_decode_each", "vd_decode_tc", "vd_decode_host", "vd_decode_radix", "vd_int_peak", "vd_transmit", "vd_transmit_bytes", "transmit", "vd_get_tune", "vd_decode_noalloc", "vd_noalloc_scratch_limit", "vd_sync", "vd_num_frames", "vd_num_kept", "vd_scratch_bytes", "vd_release_scratch",
+    "vd_server_destroy", "vd_server_replay", "vd_server_submit_device", "vd_server_submit_many", "vd_bm_gate", "vd_decode_each", "vd_decode_tc", "vd_decode_host", "vd_decode_radix", "vd_int_peak", "vd_transmit", "vd_transmit_bytes", "transmit", "vd_get_tune", "VdShape", "vd_decode_shape", "VD_FORM_PERSISTENT",
+    "VD_FORM_ONE_WAVE", "VD_FORM_FEW_FRAMES", "VD_FORM_SEGMENTS", "vd_decode_noalloc", "vd_noalloc_scratch_limit", "vd_sync", "vd_num_frames", "vd_num_kept", "vd_scratch_bytes", "vd_release_scratch",
     "vd_last_error", "vd_version", "Code", "decode",
 ]
 
 VD_OK, VD_EINVAL, VD_ENOMEM, VD_ECUDA, VD_EUNSUPPORTED, VD_ETIMEOUT, VD_EBOUNDS = 0, -1, -2, -3, -4, -5, -6
 VD_LLR_S8, VD_LLR_S4, VD_LLR_F16, VD_LLR_HARD = 0, 1, 2, 3
 VD_TERMINATED, VD_START_UNKNOWN = 1, 2
+VD_FORM_PERSISTENT, VD_FORM_ONE_WAVE, VD_FORM_FEW_FRAMES, VD_FORM_SEGMENTS = 1, 2, 3, 4
 
 _STATUS = {0: "VD_OK", -1: "VD_EINVAL", -2: "VD_ENOMEM", -3: "VD_ECUDA", -4: "VD_EUNSUPPORTED",
            -5: "VD_ETIMEOUT", -6: "VD_EBOUNDS"}
@@ -47,6 +49,12 @@ class VdTune(ctypes.Structure):
     _fields_ = [("f", ctypes.c_int32), ("v", ctypes.c_int32), ("radix", ctypes.c_int32),
                 ("lanes", ctypes.c_int32), ("threads", ctypes.c_int32),
                 ("form", ctypes.c_int32), ("reserved", ctypes.c_int32 * 2)]
+
+
+class VdShape(ctypes.Structure):
+    _fields_ = [("form", ctypes.c_int32), ("radix", ctypes.c_int32), ("lanes", ctypes.c_int32),
+                ("warp_pairs", ctypes.c_int32), ("blocks", ctypes.c_int64), ("blocks_per_sm", ctypes.c_int32),
+                ("cluster", ctypes.c_int32), ("reserved", ctypes.c_int32 * 4)]
 
 
 class VdPacket(ctypes.Structure):
@@ -164,6 +172,8 @@ def lib():
         L.vd_server_submit_many.restype = i32
         L.vd_get_tune.argtypes = [vp, i32, i32, i32, i32, P(VdTune)]
         L.vd_get_tune.restype = i32
+        L.vd_decode_shape.argtypes = [vp, i32, i64, i32, i32, i32, u32, P(VdTune), P(VdShape)]
+        L.vd_decode_shape.restype = i32
         L.vd_bm_gate.argtypes = [i32, vp, i64, i32, vp, vp, vp]
         L.vd_bm_gate.restype = i32
         L.vd_decode_host.argtypes = [vp, i32, P(vp), i32, i64, i32, i32, i32, u32, P(vp), vp]
@@ -337,11 +347,20 @@ def transmit(code, bits_words, n_info, sigma, seed, stream_id=0, terminated=Fals
 
 
 def vd_get_tune(handle, llr_type, f, v, radix) -> "VdTune":
-    """The kernel configuration vd_decode uses with tune=None."""
+    """A shape of vd_decode for streams of many frames, as a VdTune; vd_decode_shape
+    tells what runs for a stream."""
     t = VdTune()
     _check(lib().vd_get_tune(ctypes.c_void_p(handle), int(llr_type), int(f), int(v), int(radix),
                              ctypes.byref(t)))
     return t
+
+
+def vd_decode_shape(handle, llr_type, n_info, f, v, radix=2, flags=0, tune=None) -> "VdShape":
+    """What vd_decode runs for these arguments on the current device."""
+    s = VdShape()
+    _check(lib().vd_decode_shape(ctypes.c_void_p(handle), int(llr_type), int(n_info), int(f), int(v), int(radix),
+                                 int(flags), ctypes.byref(tune) if tune is not None else None, ctypes.byref(s)))
+    return s
 
 
 def vd_release_scratch() -> None:

@@ -119,6 +119,8 @@ cudaError_t launch_s(const SplitParams &p, int ranks, size_t smem, cudaStream_t 
 
 }  // namespace
 
+int wide_lanes(int K) { return K == 7 ? WideOf<7>::L : WideOf<9>::L; }
+
 bool split_plan(int K, const WideParams &in, int n_sm, SplitParams *out, int *ranks, size_t *smem) {
     return K == 7 ? split<7>(in, n_sm, out, ranks, smem) : K == 9 ? split<9>(in, n_sm, out, ranks, smem) : false;
 }

@@ -523,6 +523,33 @@ extern "C" int64_t vd_scratch_bytes(const vd_code *c, int64_t n_info, int f, int
     return (int64_t)pl.surv_bytes + extra;
 }
 
+extern "C" vd_status vd_decode_shape(const vd_code *c, int llr_type, int64_t n_info, int f, int v, int radix,
+                                     uint32_t flags, const vd_tune *tune, vd_shape *out) {
+    static const uint32_t some = 0;   // check_decode_args wants buffers
+    if (!out) return fail(VD_EINVAL, "NULL argument");
+    memset(out, 0, sizeof *out);
+    const vd_status st = check_decode_args(c, &some, llr_type, n_info, f, v, radix, flags, &some);
+    if (st != VD_OK) return st;
+    if (n_info == 0) return fail(VD_EINVAL, "an empty stream runs nothing");
+    const bool f32 = llr_type == VD_LLR_F16;
+    if (f32 && c->punctured) return fail(VD_EUNSUPPORTED, "fp16 LLRs of punctured codes are not supported");
+    Plan pl;
+    const vd_status made = make_plan(c, n_info, f, v, radix, flags, tune, &pl, f32);
+    if (made != VD_OK) return made;
+    const bool few = pl.form == Form::WIDE || pl.form == Form::SPLIT;
+    out->form = pl.form == Form::PERSISTENT ? VD_FORM_PERSISTENT
+                : pl.form == Form::WAVE     ? VD_FORM_ONE_WAVE
+                : pl.form == Form::WIDE     ? VD_FORM_FEW_FRAMES
+                                            : VD_FORM_SEGMENTS;
+    out->radix = !few && pl.r4 ? 4 : 2;
+    out->lanes = few ? vd::wide_lanes(c->K) : pl.threads_per_pair;
+    out->warp_pairs = pl.form == Form::WIDE && !pl.wide_full ? 1 : 32 / out->lanes;
+    out->blocks = pl.form == Form::SPLIT ? pl.n_win * pl.ranks : pl.blocks;
+    if (!few && !f32) out->blocks_per_sm = blocks_per_sm(pl.form == Form::PERSISTENT, c->K, pl.lanes, pl.r4);
+    out->cluster = pl.form == Form::SPLIT ? pl.ranks : 1;
+    return VD_OK;
+}
+
 extern "C" vd_status vd_decode(const vd_code *c, const void *d_llr, int llr_type, int64_t n_info,
                                int f, int v, int radix, uint32_t flags, uint32_t *d_out, int32_t *d_pm,
                                const vd_tune *tune, void *stream) {

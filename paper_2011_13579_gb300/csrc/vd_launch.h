@@ -47,6 +47,7 @@ cudaError_t stream_wave_occupancy(int K, int lanes, bool radix4, int *blocks_per
 // blocks of one warp and how much shared memory each takes; false if a
 // frame pair's survivors do not fit.
 constexpr size_t kWideSmemMax = 226u * 1024u;
+int wide_lanes(int K);   // lanes per pair of the wide and the split form
 bool wide_plan(int K, const WideParams &in, WideParams *out, int64_t *blocks, size_t *smem, bool *full);
 cudaError_t launch_wide(int K, const WideParams &p, int64_t blocks, size_t smem, bool full, cudaStream_t st);
 
