@@ -1,0 +1,69 @@
+"""Each form of vd_decode that a stream's length can lead to, by name of the
+form (vd_decode_shape), against the CPU oracle: bits and canonical final
+metrics, equal or wrong.
+
+Few frames over many lanes (wide): frames of ordinary length beyond the
+segmented form's limit of frames, with a warp's pairs full, one more, two
+more and one less, and frames so long that a warp takes one pair.
+"""
+import os
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import oracle  # noqa: E402
+import paper_2011_13579_gb300 as vd  # noqa: E402
+from paper_2011_13579_gb300 import synth  # noqa: E402
+
+GENS = {7: synth.K7_GENS, 9: synth.K9_GENS}
+THREADS = max(1, len(os.sched_getaffinity(0)))
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    vd.build()
+    yield
+
+
+def compare(K, n, f, v, term, unknown, seed, radix=2, tune=None, erase=0.0):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    code, beta = vd.Code(K, GENS[K]), len(GENS[K])
+    q = synth.make_stream(rng, K, GENS[K], n, 2.0, term).s8()
+    q[rng.random(q.size) < erase] = 0
+    out = torch.full(((n + 31) // 32,), -1, dtype=torch.int32, device="cuda")
+    pm = torch.full((vd.vd_num_frames(n, f), 1 << (K - 1)), -1, dtype=torch.int32, device="cuda")
+    flags = (vd.VD_TERMINATED if term else 0) | (vd.VD_START_UNKNOWN if unknown else 0)
+    vd.vd_decode(code.handle, torch.from_numpy(q.view(np.uint8)).cuda(), vd.VD_LLR_S8, n, f, v, radix, flags, out, pm, tune)
+    vd.vd_sync()
+    ow, opm = oracle.decode(oracle.Code(K, GENS[K]), q.reshape(-1, beta).astype(np.int32), n, f, v, terminated=term,
+                            start_unknown=unknown, threads=THREADS, want_pm=True)
+    assert np.array_equal(out.cpu().numpy().view(np.uint32), ow), (n, f, v)
+    assert np.array_equal(pm.cpu().numpy().astype(np.int64), opm), (n, f, v)   # every frame has K-1 stages or more
+    return vd.vd_decode_shape(code.handle, vd.VD_LLR_S8, n, f, v, radix, flags, tune)
+
+
+# K, f, v, the segmented form's frames per SM at that length, pairs per warp
+WIDE = [(7, 256, 42, 2, 4), (7, 512, 42, 3, 4), (7, 2560, 42, 3, 1), (7, 8192, 42, 3, 1), (9, 512, 64, 3, 1), (9, 96, 64, 1, 1)]
+
+
+@pytest.mark.parametrize("term,unknown", [(True, False), (False, True)])
+@pytest.mark.parametrize("K,f,v,frames_per_sm,warp_pairs", WIDE)
+def test_wide_form_beyond_the_segmented_one(K, f, v, frames_per_sm, warp_pairs, term, unknown):
+    limit = frames_per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    first = -(-(limit + 1) // 8) * 8           # frames of a whole number of warps
+    for extra in (0, 1, 2, 7) if f <= 512 else (1,):
+        n = (first + extra - 1) * f + 45       # the last frame is a short one
+        s = compare(K, n, f, v, term, unknown, seed=n + K + term, erase=0.3 if extra == 2 else 0.0)
+        assert (s.form, s.warp_pairs) == (vd.VD_FORM_FEW_FRAMES, warp_pairs), (n, s.form, s.warp_pairs)
+
+
+def test_forms_around_the_segmented_limit():
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    code = vd.Code(7, GENS[7])
+    forms = [vd.vd_decode_shape(code.handle, vd.VD_LLR_S8, frames * 256, 256, 42).form for frames in (1, 2 * sm, 2 * sm + 1)]
+    assert forms == [vd.VD_FORM_SEGMENTS, vd.VD_FORM_SEGMENTS, vd.VD_FORM_FEW_FRAMES]
