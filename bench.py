@@ -188,6 +188,18 @@ def whole_job_value(ms_local, bits_per_rank_step, steps, world, device=None):
     return ms, bits_per_rank_step * steps * world / (ms / 1e3) / 1e9
 
 
+def named_tune(vd, radix, lanes, code_k=K):
+    """The vd_tune of a vd_decode call that is to run the radix (and lanes) named:
+    left open, the library runs a K=7 stream in radix-2 steps, so radix 4 names a lane there."""
+    if not lanes and radix == 4 and code_k == 7:
+        lanes = 1
+    if not lanes:
+        return None
+    tune = vd.VdTune()
+    tune.lanes = lanes
+    return tune
+
+
 def run_gpu(args, rank, world):
     import torch
     import torch.distributed as dist
@@ -207,13 +219,10 @@ def run_gpu(args, rank, world):
     llr_dev = [arena[i * BETA * N_INFO:(i + 1) * BETA * N_INFO] for i in range(len(streams))]
     outs = [out_arena[i * nw:(i + 1) * nw] for i in range(len(streams))]
     s = torch.cuda.Stream(dev)
-    tune = None
-    if args.lanes:
-        tune = vd.VdTune()
-        tune.lanes = args.lanes
+    tune = named_tune(vd, args.radix, args.lanes)
     flags = 0
     plan = stream_plan(vd, code, len(streams), args.radix, args.lanes, s) if args.path == "batch" else None
-    shape = {"radix": args.radix, "lanes": args.lanes}
+    shape = {"radix": args.radix, "lanes": tune.lanes if tune else 0}
     if plan is not None:
         info = plan.info()   # lanes chosen by the plan's measured autotuner when --lanes is 0
         shape = {"radix": int(info.radix), "lanes": int(info.lanes)}
@@ -891,10 +900,7 @@ def kernel_only(args):
             st, f, v = synth.segmented_stream(3.0), F, V
         llr = torch.from_numpy(st.s8().view(np.uint8)).cuda()
         out = torch.empty(N_INFO // 32, dtype=torch.int32, device="cuda")
-        tune = None
-        if args.lanes:
-            tune = vd.VdTune()
-            tune.lanes = args.lanes
+        tune = named_tune(vd, args.radix, args.lanes, code.K)
         for _ in range(args.warmup + args.steps):
             vd.vd_decode(code.handle, llr, vd.VD_LLR_S8, N_INFO, f, v, args.radix, 0, out, None, tune, None)
         torch.cuda.synchronize()

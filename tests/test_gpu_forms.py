@@ -2,9 +2,10 @@
 form (vd_decode_shape), against the CPU oracle: bits and canonical final
 metrics, equal or wrong.
 
-Few frames over many lanes (wide): frames of ordinary length beyond the
-segmented form's limit of frames, with a warp's pairs full, one more, two
-more and one less, and frames so long that a warp takes one pair.
+* few frames over many lanes (wide): frames of ordinary length beyond the
+  segmented form's limit of frames, with a warp's pairs full, one more, two
+  more and one less, and frames so long that a warp takes one pair;
+* radix 4, which runs only where the caller names lanes or a form (K=7).
 """
 import os
 
@@ -67,3 +68,21 @@ def test_forms_around_the_segmented_limit():
     code = vd.Code(7, GENS[7])
     forms = [vd.vd_decode_shape(code.handle, vd.VD_LLR_S8, frames * 256, 256, 42).form for frames in (1, 2 * sm, 2 * sm + 1)]
     assert forms == [vd.VD_FORM_SEGMENTS, vd.VD_FORM_SEGMENTS, vd.VD_FORM_FEW_FRAMES]
+
+
+@pytest.mark.parametrize("form", [vd.VD_FORM_PERSISTENT, vd.VD_FORM_ONE_WAVE])
+@pytest.mark.parametrize("K,lanes", [(7, 1), (7, 2), (7, 4), (9, 4), (9, 8)])
+def test_radix_4_in_both_named_forms(K, lanes, form):
+    t = vd.VdTune()
+    t.lanes, t.form = lanes, form
+    f, v = (256, 42) if K == 7 else (512, 64)
+    s = compare(K, 150_777, f, v, True, False, seed=600 + K + lanes, radix=4, tune=t)
+    assert (s.form, s.radix, s.lanes) == (form, 4, lanes)
+
+
+def test_radix_4_persistent_with_several_tasks_a_warp():
+    t = vd.VdTune()
+    t.lanes, t.form = 1, vd.VD_FORM_PERSISTENT
+    n, f = (1 << 22) + 77, 32                  # 2049 tasks of 32 pairs
+    s = compare(7, n, f, 8, False, False, seed=66, radix=4, tune=t)
+    assert s.radix == 4 and (vd.vd_num_frames(n, f) + 63) // 64 > s.blocks * 4
