@@ -370,10 +370,23 @@ int blocks_per_sm(bool persistent, int K, int lanes, bool r4) {
 // 4.2 M (1.9 waves) 56 / 67, 8.4 M (3.9) 103 / 99; K=9, f = 512: 10^5 bits 44 / 136,
 // 10^6 (1.3) 83 / 136, 2.1 M (2.6) 130 / 136, 3 M (3.9) 199 / 188.
 constexpr double kWideWavesK7 = 3.5, kWideWavesK9 = 2.6;
+// Frames of up to about 100 stages take so little shared memory that the warps
+// per SM, not the waves, say when the lanes' extra instructions outweigh the shorter
+// chain.  Measured (us, wide / the next form, at so many blocks per SM): K=7, f = 32, v = 6: 32
+// 23.0 / 23.2, 45 29.2 / 23.2, 64 38.4 / 38.4, 77 44.5 / 38.7; f = 64, v = 30: 38 47.7 / 51.7, 45 56.0 /
+// 51.6, 64 77.6 / 82.6, 77 about equal (the next form is one wave up to 64 blocks, persistent beyond);
+// K=9, f = 32, v = 6: 20 19.8 / 19.1, 31 25.2 / 21.1, 62 45.6 / 33.2; f = 192, v = 42: 21 80.4 / 88.6, 26 92.8 / 88.8.
+constexpr int64_t kWideBlocksK7 = 38, kWideBlocksK7Persistent = 70, kWideBlocksK9 = 24;
 
-bool take_wide(int K, int64_t blocks, size_t smem) {
+// One lane per pair in one wave of two warps per scheduler (choose_shape).
+bool one_lane_wave(int64_t n_pairs) { return (n_pairs + 31) / 32 <= 2 * 4 * (int64_t)sm_count(); }
+
+bool take_wide(int K, int64_t n_pairs, int64_t blocks, size_t smem) {
+    const int64_t n_sm = sm_count();
     const int64_t per_sm = (int64_t)((228u * 1024u) / (smem + 1024u));   // 228 KB an SM, 1 KB of it reserved per block
-    return (double)blocks <= (K == 7 ? kWideWavesK7 : kWideWavesK9) * (double)(sm_count() * std::max<int64_t>(1, per_sm));
+    const int64_t most = K == 9 ? kWideBlocksK9 : one_lane_wave(n_pairs) ? kWideBlocksK7 : kWideBlocksK7Persistent;
+    return (double)blocks <= (K == 7 ? kWideWavesK7 : kWideWavesK9) * (double)(n_sm * std::max<int64_t>(1, per_sm)) &&
+           blocks <= most * n_sm;
 }
 
 size_t wave_scratch(int64_t n_pairs, int lanes, int64_t wmax, const vd::KernelGeom &g, int64_t *blocks) {
@@ -397,7 +410,7 @@ void choose_shape(const vd_code *c, bool r4, int64_t n_pairs, int64_t wmax, int 
     auto resident_pairs = [&](int l) { return n_sm * blocks_per_sm(false, c->K, l, r4) * (vd::kThreads / l); };
     if (c->kind == vd::KIND_K7_R2) {
         *lanes = n_pairs <= resident_pairs(2) ? 2 : 1;
-        const bool fits = *lanes == 2 || (n_pairs + 31) / 32 <= 2 * 4 * n_sm;
+        const bool fits = *lanes == 2 || one_lane_wave(n_pairs);
         *form = fits || n_sm * blocks_per_sm(true, c->K, *lanes, r4) < 1 ? Form::WAVE : Form::PERSISTENT;
         return;
     }
@@ -461,7 +474,7 @@ vd_status make_plan(const vd_code *c, int64_t n_info, int f, int v, int radix, u
             return VD_OK;
         }
         if (vd::wide_plan(c->K, wp, &pl->wide, &pl->blocks, &pl->smem, &pl->wide_full) &&
-            take_wide(c->K, pl->blocks, pl->smem)) {
+            take_wide(c->K, pl->n_pairs, pl->blocks, pl->smem)) {
             pl->form = Form::WIDE;
             return VD_OK;
         }

@@ -70,6 +70,16 @@ def test_forms_around_the_segmented_limit():
     assert forms == [vd.VD_FORM_SEGMENTS, vd.VD_FORM_SEGMENTS, vd.VD_FORM_FEW_FRAMES]
 
 
+@pytest.mark.parametrize("K,f,v,per_sm,few", [(7, 32, 6, 37, True), (7, 32, 6, 42, False), (7, 64, 30, 37, True),
+                                              (7, 64, 30, 46, False), (7, 32, 6, 80, False), (9, 32, 6, 23, True),
+                                              (9, 32, 6, 60, False), (9, 64, 30, 40, False)])
+def test_short_frames_leave_the_wide_form_by_blocks_per_sm(K, f, v, per_sm, few):
+    """per_sm: blocks of the wide form (four pairs for K=7, one for K=9) per SM."""
+    n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count * (8 if K == 7 else 2) * f
+    s = compare(K, n, f, v, True, False, seed=n)
+    assert (s.form == vd.VD_FORM_FEW_FRAMES) == few, s.form
+
+
 @pytest.mark.parametrize("form", [vd.VD_FORM_PERSISTENT, vd.VD_FORM_ONE_WAVE])
 @pytest.mark.parametrize("K,lanes", [(7, 1), (7, 2), (7, 4), (9, 4), (9, 8)])
 def test_radix_4_in_both_named_forms(K, lanes, form):
