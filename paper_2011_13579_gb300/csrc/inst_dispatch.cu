@@ -4,16 +4,16 @@
 
 namespace vd {
 
-cudaError_t launch_stream_k7(int lanes, bool radix4, const StreamParams &p, int64_t blocks,
+cudaError_t launch_stream_k7(int lanes, bool radix4, const StreamParams &p, int64_t blocks, bool deep,
                              cudaStream_t st) {
-#define X(K, R4, L) if (K == 7 && radix4 == R4 && lanes == L) return launch_stream_v<K, R4, L>(p, blocks, st);
+#define X(K, R4, L) if (K == 7 && radix4 == R4 && lanes == L) return launch_stream_v<K, R4, L>(p, blocks, deep, st);
     VD_VARIANT_LIST(X)
 #undef X
     return cudaErrorInvalidValue;
 }
-cudaError_t launch_stream_k9(int lanes, bool radix4, const StreamParams &p, int64_t blocks,
+cudaError_t launch_stream_k9(int lanes, bool radix4, const StreamParams &p, int64_t blocks, bool deep,
                              cudaStream_t st) {
-#define X(K, R4, L) if (K == 9 && radix4 == R4 && lanes == L) return launch_stream_v<K, R4, L>(p, blocks, st);
+#define X(K, R4, L) if (K == 9 && radix4 == R4 && lanes == L) return launch_stream_v<K, R4, L>(p, blocks, deep, st);
     VD_VARIANT_LIST(X)
 #undef X
     return cudaErrorInvalidValue;
@@ -60,8 +60,9 @@ cudaError_t stream_persistent_occupancy(int K, int lanes, bool radix4, int *bloc
     return cudaErrorInvalidValue;
 }
 
-cudaError_t stream_wave_occupancy(int K, int lanes, bool radix4, int *blocks_per_sm) {
-#define X(KK, R4, L) if (K == KK && radix4 == R4 && lanes == L) return occupancy_wave_v<KK, R4, L>(blocks_per_sm);
+cudaError_t stream_wave_occupancy(int K, int lanes, bool radix4, bool deep, int *blocks_per_sm) {
+#define X(KK, R4, L) \
+    if (K == KK && radix4 == R4 && lanes == L) return occupancy_wave_v<KK, R4, L>(deep, blocks_per_sm);
     VD_VARIANT_LIST(X)
 #undef X
     return cudaErrorInvalidValue;

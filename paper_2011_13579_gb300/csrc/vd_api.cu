@@ -340,23 +340,25 @@ int sm_count() {
     return cache[dev] = n;
 }
 
-// Resident blocks per SM of the persistent or the one-wave stream kernel, per
-// device and shape; 0 (and nothing kept) if the query fails.
-int blocks_per_sm(bool persistent, int K, int lanes, bool r4) {
+// Resident blocks per SM of a stream kernel, per device and shape; 0 (and
+// nothing kept) if the query fails.
+enum class Kernel { PERSISTENT, WAVE, WAVE_SHALLOW };
+int blocks_per_sm(Kernel kernel, int K, int lanes, bool r4) {
     static std::mutex mu;
-    static std::map<std::tuple<int, bool, int, int, bool>, int> cache;
+    static std::map<std::tuple<int, Kernel, int, int, bool>, int> cache;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     std::lock_guard<std::mutex> lk(mu);
-    const auto key = std::make_tuple(dev, persistent, K, lanes, r4);
+    const auto key = std::make_tuple(dev, kernel, K, lanes, r4);
     auto it = cache.find(key);
     if (it != cache.end()) return it->second;
     int bps = 0;
-    if ((persistent ? vd::stream_persistent_occupancy(K, lanes, r4, &bps)
-                    : vd::stream_wave_occupancy(K, lanes, r4, &bps)) != cudaSuccess) {
+    if ((kernel == Kernel::PERSISTENT ? vd::stream_persistent_occupancy(K, lanes, r4, &bps)
+                                      : vd::stream_wave_occupancy(K, lanes, r4, kernel == Kernel::WAVE, &bps)) !=
+        cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -373,20 +375,16 @@ constexpr double kWideWavesK7 = 3.5, kWideWavesK9 = 2.6;
 // Frames of up to about 100 stages take so little shared memory that the warps
 // per SM, not the waves, say when the lanes' extra instructions outweigh the shorter
 // chain.  Measured (us, wide / the next form, at so many blocks per SM): K=7, f = 32, v = 6: 32
-// 23.0 / 23.2, 45 29.2 / 23.2, 64 38.4 / 38.4, 77 44.5 / 38.7; f = 64, v = 30: 38 47.7 / 51.7, 45 56.0 /
-// 51.6, 64 77.6 / 82.6, 77 about equal (the next form is one wave up to 64 blocks, persistent beyond);
-// K=9, f = 32, v = 6: 20 19.8 / 19.1, 31 25.2 / 21.1, 62 45.6 / 33.2; f = 192, v = 42: 21 80.4 / 88.6, 26 92.8 / 88.8.
-constexpr int64_t kWideBlocksK7 = 38, kWideBlocksK7Persistent = 70, kWideBlocksK9 = 24;
+// 23.0 / 23.2, 45 29.2 / 23.2, 64 38.4 / 35.8, 77 44.5 / 36.0; f = 64, v = 30: 38 47.7 / 51.7, 45 56.0 /
+// 51.6, 64 77.6 / 79.4, 84 96 / 82.9; K=9, f = 32, v = 6: 20 19.8 / 19.1, 31 25.2 / 21.1, 62 45.6 / 33.2; f = 192,
+// v = 42: 21 80.4 / 88.6, 26 92.8 / 88.8.
+constexpr int64_t kWideBlocksK7 = 38, kWideBlocksK9 = 24;
 
-// One lane per pair in one wave of two warps per scheduler (choose_shape).
-bool one_lane_wave(int64_t n_pairs) { return (n_pairs + 31) / 32 <= 2 * 4 * (int64_t)sm_count(); }
-
-bool take_wide(int K, int64_t n_pairs, int64_t blocks, size_t smem) {
+bool take_wide(int K, int64_t blocks, size_t smem) {
     const int64_t n_sm = sm_count();
     const int64_t per_sm = (int64_t)((228u * 1024u) / (smem + 1024u));   // 228 KB an SM, 1 KB of it reserved per block
-    const int64_t most = K == 9 ? kWideBlocksK9 : one_lane_wave(n_pairs) ? kWideBlocksK7 : kWideBlocksK7Persistent;
     return (double)blocks <= (K == 7 ? kWideWavesK7 : kWideWavesK9) * (double)(n_sm * std::max<int64_t>(1, per_sm)) &&
-           blocks <= most * n_sm;
+           blocks <= (K == 7 ? kWideBlocksK7 : kWideBlocksK9) * n_sm;
 }
 
 size_t wave_scratch(int64_t n_pairs, int lanes, int64_t wmax, const vd::KernelGeom &g, int64_t *blocks) {
@@ -396,9 +394,10 @@ size_t wave_scratch(int64_t n_pairs, int lanes, int64_t wmax, const vd::KernelGe
 
 // Lanes per pair and form of a stream too long for the forms above, when the
 // caller leaves both open (us per call at the stated bits, f = 256 or 512).
-// K=7: two lanes per pair while all pairs are resident (10 M: 132 against 157
-// with one); one lane while no scheduler has more than two warps (16.8 M: 159
-// against 187); then the persistent form (20 M: 217 against 241).
+// K=7: two lanes per pair while all pairs are resident (10 M: 129 against 154
+// with one); one lane while they are, three blocks per SM with the shallow ring (16.8 M: 159 against 183;
+// 20 M 211, 29 M 221 against 215 and 224 with the persistent form; f = 32, 3 M: 36.0 against 38.5); then the
+// persistent form.
 // K=9: eight lanes while all pairs are resident (4.2 M: 188 against 283 with four), then four
 // while they are (8.4 M: 314 against 362), then eight again (10 M 437 / 532,
 // 16.8 M 590 / 621, 20 M 739 / 801 against the persistent form with four) while
@@ -407,24 +406,26 @@ size_t wave_scratch(int64_t n_pairs, int lanes, int64_t wmax, const vd::KernelGe
 // known, or zero, the one-wave form runs.
 void choose_shape(const vd_code *c, bool r4, int64_t n_pairs, int64_t wmax, int *lanes, Form *form) {
     const int64_t n_sm = sm_count();
-    auto resident_pairs = [&](int l) { return n_sm * blocks_per_sm(false, c->K, l, r4) * (vd::kThreads / l); };
+    auto resident_pairs = [&](int l, Kernel kernel) {
+        return n_sm * blocks_per_sm(kernel, c->K, l, r4) * (vd::kThreads / l);
+    };
     if (c->kind == vd::KIND_K7_R2) {
-        *lanes = n_pairs <= resident_pairs(2) ? 2 : 1;
-        const bool fits = *lanes == 2 || one_lane_wave(n_pairs);
-        *form = fits || n_sm * blocks_per_sm(true, c->K, *lanes, r4) < 1 ? Form::WAVE : Form::PERSISTENT;
+        *lanes = n_pairs <= resident_pairs(2, Kernel::WAVE) ? 2 : 1;
+        const bool fits = *lanes == 2 || n_pairs <= resident_pairs(1, Kernel::WAVE_SHALLOW);
+        *form = fits || n_sm * blocks_per_sm(Kernel::PERSISTENT, c->K, *lanes, r4) < 1 ? Form::WAVE : Form::PERSISTENT;
         return;
     }
     *form = Form::WAVE;
     *lanes = 8;
-    if (n_pairs <= resident_pairs(8)) return;
-    if (n_pairs <= resident_pairs(4)) {
+    if (n_pairs <= resident_pairs(8, Kernel::WAVE)) return;
+    if (n_pairs <= resident_pairs(4, Kernel::WAVE)) {
         *lanes = 4;
         return;
     }
     vd::KernelGeom g8, g4;
     int64_t blocks = 0;
     if (!geometry(c->kind, 8, r4, &g8) || !geometry(c->kind, 4, r4, &g4)) return;
-    const size_t persistent = 2u * (size_t)(n_sm * blocks_per_sm(true, c->K, 4, r4)) * vd::kThreads *
+    const size_t persistent = 2u * (size_t)(n_sm * blocks_per_sm(Kernel::PERSISTENT, c->K, 4, r4)) * vd::kThreads *
                               (size_t)((wmax + g4.U - 1) / g4.U * g4.U) * g4.NW * 4u;
     if (persistent > 0 && wave_scratch(n_pairs, 8, wmax, g8, &blocks) > persistent) {
         *lanes = 4;
@@ -474,7 +475,7 @@ vd_status make_plan(const vd_code *c, int64_t n_info, int f, int v, int radix, u
             return VD_OK;
         }
         if (vd::wide_plan(c->K, wp, &pl->wide, &pl->blocks, &pl->smem, &pl->wide_full) &&
-            take_wide(c->K, pl->n_pairs, pl->blocks, pl->smem)) {
+            take_wide(c->K, pl->blocks, pl->smem)) {
             pl->form = Form::WIDE;
             return VD_OK;
         }
@@ -488,7 +489,7 @@ vd_status make_plan(const vd_code *c, int64_t n_info, int f, int v, int radix, u
         // the caller's lanes; the persistent form from a task per resident warp up
         pl->threads_per_pair = pl->lanes;
         const int64_t tasks = (pl->n_pairs + 32 / pl->lanes - 1) / (32 / pl->lanes);
-        const int64_t warps = (int64_t)sm_count() * blocks_per_sm(true, c->K, pl->lanes, pl->r4) * (vd::kThreads / 32);
+        const int64_t warps = (int64_t)sm_count() * blocks_per_sm(Kernel::PERSISTENT, c->K, pl->lanes, pl->r4) * (vd::kThreads / 32);
         if (warps > 0 && (form == 1 || (form == 0 && tasks >= warps))) pl->form = Form::PERSISTENT;
     }
     const int64_t wpad = ((wmax + pl->geom.U - 1) / pl->geom.U) * pl->geom.U;
@@ -498,7 +499,7 @@ vd_status make_plan(const vd_code *c, int64_t n_info, int f, int v, int radix, u
     if (pl->form == Form::PERSISTENT) {
         // resident warps pull tasks and hide each task's traceback behind the
         // next task's forward pass; each owns two survivor buffers
-        pl->blocks = (int64_t)sm_count() * blocks_per_sm(true, c->K, pl->lanes, pl->r4);
+        pl->blocks = (int64_t)sm_count() * blocks_per_sm(Kernel::PERSISTENT, c->K, pl->lanes, pl->r4);
         pl->surv_bytes = 2u * (size_t)pl->blocks * vd::kThreads * (size_t)wpad * pl->geom.NW * 4u;
     } else {
         pl->surv_bytes = wave_scratch(pl->n_pairs, pl->threads_per_pair, wmax, pl->geom, &pl->blocks);
@@ -525,6 +526,10 @@ vd_status check_decode_args(const vd_code *c, const void *d_llr, int llr_type, i
 }
 
 }  // namespace
+
+bool vd_internal_wave_deep(int K, int lanes, bool r4, int64_t blocks) {
+    return blocks <= (int64_t)sm_count() * blocks_per_sm(Kernel::WAVE, K, lanes, r4);
+}
 
 extern "C" int64_t vd_scratch_bytes(const vd_code *c, int64_t n_info, int f, int v, int radix,
                                     const vd_tune *tune) {
@@ -558,7 +563,12 @@ extern "C" vd_status vd_decode_shape(const vd_code *c, int llr_type, int64_t n_i
     out->lanes = few ? vd::wide_lanes(c->K) : pl.threads_per_pair;
     out->warp_pairs = pl.form == Form::WIDE && !pl.wide_full ? 1 : 32 / out->lanes;
     out->blocks = pl.form == Form::SPLIT ? pl.n_win * pl.ranks : pl.blocks;
-    if (!few && !f32) out->blocks_per_sm = blocks_per_sm(pl.form == Form::PERSISTENT, c->K, pl.lanes, pl.r4);
+    if (!few && !f32) {
+        const Kernel kernel = pl.form == Form::PERSISTENT ? Kernel::PERSISTENT
+                              : vd_internal_wave_deep(c->K, pl.lanes, pl.r4, pl.blocks) ? Kernel::WAVE
+                                                                                       : Kernel::WAVE_SHALLOW;
+        out->blocks_per_sm = blocks_per_sm(kernel, c->K, pl.lanes, pl.r4);
+    }
     out->cluster = pl.form == Form::SPLIT ? pl.ranks : 1;
     return VD_OK;
 }
@@ -656,14 +666,15 @@ extern "C" vd_status vd_decode(const vd_code *c, const void *d_llr, int llr_type
         if (e != cudaSuccess) return cuda_fail(e, "decode launch");
         return VD_OK;
     }
+    const bool deep = !f32 && vd_internal_wave_deep(c->K, pl.lanes, pl.r4, pl.blocks);
     switch (c->kind) {
     case vd::KIND_K7_R2:
         e = f32 ? vd::launch_stream_f32(c->K, pl.threads_per_pair, p, pl.blocks, cs)
-                : vd::launch_stream_k7(pl.lanes, pl.r4, p, pl.blocks, cs);
+                : vd::launch_stream_k7(pl.lanes, pl.r4, p, pl.blocks, deep, cs);
         break;
     case vd::KIND_K9_R3:
         e = f32 ? vd::launch_stream_f32(c->K, pl.threads_per_pair, p, pl.blocks, cs)
-                : vd::launch_stream_k9(pl.lanes, pl.r4, p, pl.blocks, cs);
+                : vd::launch_stream_k9(pl.lanes, pl.r4, p, pl.blocks, deep, cs);
         break;
     default: return fail(VD_EUNSUPPORTED, "no kernel for this code");
     }

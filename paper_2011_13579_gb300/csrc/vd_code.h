@@ -29,6 +29,9 @@ vd_status vd_internal_noalloc_status(void);
 // use; NULL if it cannot be allocated), for kernels outside vd_api.cu.
 int *vd_internal_status_word(void);
 
+// Whether every block of a one-wave launch is resident at once, on the current device.
+bool vd_internal_wave_deep(int K, int lanes, bool radix4, int64_t blocks);
+
 // A buffer of at least `bytes` from the library's scratch pool of the current
 // device and `stream` (slots 0-5 belong to vd_api.cu; 6 = vd_decode_radix).
 vd_status vd_internal_scratch(int slot, size_t bytes, cudaStream_t stream, void **out);

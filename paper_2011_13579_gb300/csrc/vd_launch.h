@@ -25,9 +25,10 @@ struct KernelGeom {
 };
 
 // Returns cudaErrorInvalidValue if (kind, lanes, radix4) has no instantiation.
-cudaError_t launch_stream_k7(int lanes, bool radix4, const StreamParams &p, int64_t blocks,
+// deep: the traceback ring for launches of which every block is resident at once (StreamSmem).
+cudaError_t launch_stream_k7(int lanes, bool radix4, const StreamParams &p, int64_t blocks, bool deep,
                              cudaStream_t st);
-cudaError_t launch_stream_k9(int lanes, bool radix4, const StreamParams &p, int64_t blocks,
+cudaError_t launch_stream_k9(int lanes, bool radix4, const StreamParams &p, int64_t blocks, bool deep,
                              cudaStream_t st);
 cudaError_t launch_batch_k7(int lanes, bool radix4, const BatchParams &p, int64_t blocks,
                             cudaStream_t st);
@@ -40,7 +41,7 @@ cudaError_t launch_stream_persistent(int K, int lanes, bool radix4, const Stream
                                      cudaStream_t st);
 cudaError_t stream_persistent_occupancy(int K, int lanes, bool radix4, int *blocks_per_sm);
 // The same for the kernel with one lane group per frame pair (launch_stream_k7 / _k9).
-cudaError_t stream_wave_occupancy(int K, int lanes, bool radix4, int *blocks_per_sm);
+cudaError_t stream_wave_occupancy(int K, int lanes, bool radix4, bool deep, int *blocks_per_sm);
 
 // Wide form (vd_wide.cuh), for streams of few frames: wide_plan fills the
 // padded length, the records kept and the pairs per warp, and says how many

@@ -173,8 +173,9 @@ extern "C" vd_status vd_decode_noalloc(const vd_code *c, const void *d_llr, int6
     p.status = status;
     p.counter = nullptr;   // the non-persistent kernel takes no task counter
     p.n_tasks = 0;
-    e = (c->kind == vd::KIND_K7_R2) ? vd::launch_stream_k7(lanes, radix == 4, p, blocks, cs)
-                                    : vd::launch_stream_k9(lanes, radix == 4, p, blocks, cs);
+    const bool deep = vd_internal_wave_deep(c->K, lanes, radix == 4, blocks);
+    e = (c->kind == vd::KIND_K7_R2) ? vd::launch_stream_k7(lanes, radix == 4, p, blocks, deep, cs)
+                                    : vd::launch_stream_k9(lanes, radix == 4, p, blocks, deep, cs);
     if (e != cudaSuccess) return fail(VD_ECUDA, "decode launch: %s", cudaGetErrorString(e));
     return VD_OK;
 }

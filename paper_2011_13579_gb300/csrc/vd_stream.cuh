@@ -1011,13 +1011,19 @@ __device__ __forceinline__ bool forward_pair(const FrameTask (&ft)[2], uint32_t 
 
 // Shared memory of the one-wave kernel (dynamic): per warp the staging of its
 // traceback, then a traceback record per thread.  Its traceback has the SM
-// to itself, so its time is the latency of the copies over the pairs in flight: two
+// to itself, so its time is the latency of the copies over the pairs in flight (DEEP): two
 // where a pair of groups takes 6 KB a warp or more (three would leave the loads of received
-// values 28 KB of L1), three otherwise.
-template <int K, int BETA, uint64_t GENS, int L, bool RADIX4, int NT>
+// values 28 KB of L1), three otherwise.  Where a pair takes 8 KB a warp (K=7 radix 2 with one
+// lane, K=9 with four) that leaves two blocks an SM.  Launches of more blocks than those hold at
+// once take the shallow form there: one pair in flight, and registers for three blocks (us, deep /
+// shallow: K=7 with one lane, 22 M bits 243 / 213, 26 M 244 / 216; K=9 with four, 10 M bits 538 / 441, 14.5 M
+// 606 / 476).
+template <int K, int BETA, uint64_t GENS, int L, bool RADIX4, int NT, bool DEEP>
 struct StreamSmem {
     using Cfg = StreamCfg<K, BETA, GENS, L, RADIX4>;
-    static constexpr int D = Traceback<K, L, RADIX4, Cfg::NR, Cfg::NW, Cfg::ES>::STAGE_WORDS * 4 >= 6144 ? 2 : 3;
+    static constexpr size_t PAIR_BYTES = Traceback<K, L, RADIX4, Cfg::NR, Cfg::NW, Cfg::ES>::STAGE_WORDS * 4u;
+    static constexpr int D = !DEEP ? 1 : PAIR_BYTES >= 6144 ? 2 : 3;
+    static constexpr bool HAS_SHALLOW = PAIR_BYTES >= 8192;
     using Tb = Traceback<K, L, RADIX4, Cfg::NR, Cfg::NW, Cfg::ES, D>;
     static constexpr size_t STG_BYTES = (size_t)(NT / 32) * Tb::STAGE_WORDS * 4u;
     static constexpr size_t BYTES = STG_BYTES + (size_t)NT * sizeof(TbState);
@@ -1025,11 +1031,11 @@ struct StreamSmem {
 };
 
 // Segmented decode of one stream: frame pair q = (2q, 2q+1) per group of L lanes.
-template <int K, int BETA, uint64_t GENS, int L, bool RADIX4, int NT>
-__global__ void __launch_bounds__(NT) stream_kernel(const StreamParams p) {
+template <int K, int BETA, uint64_t GENS, int L, bool RADIX4, int NT, bool DEEP>
+__global__ void __launch_bounds__(NT, DEEP ? 0 : 3) stream_kernel(const StreamParams p) {
     constexpr int NS = 1 << (K - 1);
     using Cfg = StreamCfg<K, BETA, GENS, L, RADIX4>;
-    using Sm = StreamSmem<K, BETA, GENS, L, RADIX4, NT>;
+    using Sm = StreamSmem<K, BETA, GENS, L, RADIX4, NT, DEEP>;
     using Tb = typename Sm::Tb;
     extern __shared__ __align__(16) uint4 vd_dyn_smem[];
     auto stg = reinterpret_cast<uint32_t (*)[Tb::STAGE_WORDS]>(vd_dyn_smem);

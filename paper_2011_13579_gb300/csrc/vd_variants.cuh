@@ -34,25 +34,43 @@ cudaError_t opt_in_smem(Kern kern, size_t bytes, std::atomic<uint64_t> &done) {
     return e;
 }
 
+// The one-wave kernel: deep or shallow traceback ring (StreamSmem), one
+// kernel where a shape has no shallow form.
+template <int K, bool R4, int L, bool DEEP>
+struct WaveKernel {
+    using Sm = StreamSmem<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads, DEEP>;
+    static constexpr auto kern = stream_kernel<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads, DEEP>;
+    static cudaError_t opt_in() {
+        static std::atomic<uint64_t> done{0};
+        return opt_in_smem(kern, Sm::BYTES, done);
+    }
+    static cudaError_t launch(const StreamParams &p, int64_t blocks, cudaStream_t st) {
+        const cudaError_t e = opt_in();
+        if (e != cudaSuccess) return e;
+        kern<<<(unsigned)blocks, kThreads, Sm::BYTES, st>>>(p);
+        return cudaGetLastError();
+    }
+    static cudaError_t occupancy(int *blocks_per_sm) {
+        const cudaError_t e = opt_in();
+        if (e != cudaSuccess) return e;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, kThreads, Sm::BYTES);
+    }
+};
+
 template <int K, bool R4, int L>
-cudaError_t launch_stream_v(const StreamParams &p, int64_t blocks, cudaStream_t st) {
-    constexpr size_t bytes = StreamSmem<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads>::BYTES;
-    static std::atomic<uint64_t> done{0};
-    const cudaError_t e = opt_in_smem(stream_kernel<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads>, bytes, done);
-    if (e != cudaSuccess) return e;
-    stream_kernel<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads>
-        <<<(unsigned)blocks, kThreads, bytes, st>>>(p);
-    return cudaGetLastError();
+cudaError_t launch_stream_v(const StreamParams &p, int64_t blocks, bool deep, cudaStream_t st) {
+    if constexpr (WaveKernel<K, R4, L, true>::Sm::HAS_SHALLOW) {
+        if (!deep) return WaveKernel<K, R4, L, false>::launch(p, blocks, st);
+    }
+    return WaveKernel<K, R4, L, true>::launch(p, blocks, st);
 }
 
 template <int K, bool R4, int L>
-cudaError_t occupancy_wave_v(int *blocks_per_sm) {
-    constexpr size_t bytes = StreamSmem<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads>::BYTES;
-    static std::atomic<uint64_t> done{0};
-    const auto kern = stream_kernel<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, R4, kThreads>;
-    const cudaError_t e = opt_in_smem(kern, bytes, done);
-    if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, kThreads, bytes);
+cudaError_t occupancy_wave_v(bool deep, int *blocks_per_sm) {
+    if constexpr (WaveKernel<K, R4, L, true>::Sm::HAS_SHALLOW) {
+        if (!deep) return WaveKernel<K, R4, L, false>::occupancy(blocks_per_sm);
+    }
+    return WaveKernel<K, R4, L, true>::occupancy(blocks_per_sm);
 }
 
 template <int K, bool R4, int L>
@@ -126,8 +144,8 @@ cudaError_t occupancy_stream_v(int *blocks_per_sm) {
     X(9, false, 4) X(9, false, 8) X(9, true, 4) X(9, true, 8)
 
 #define VD_DECLARE_VARIANT(K, R4, L)                                                           \
-    extern template cudaError_t launch_stream_v<K, R4, L>(const StreamParams &, int64_t, cudaStream_t); \
-    extern template cudaError_t occupancy_wave_v<K, R4, L>(int *);                              \
+    extern template cudaError_t launch_stream_v<K, R4, L>(const StreamParams &, int64_t, bool, cudaStream_t); \
+    extern template cudaError_t occupancy_wave_v<K, R4, L>(bool, int *);                        \
     extern template cudaError_t launch_batch_v<K, R4, L>(const BatchParams &, int64_t, cudaStream_t);   \
     extern template cudaError_t occupancy_v<K, R4, L>(int *);                                   \
     extern template cudaError_t launch_stream_persistent_v<K, R4, L>(const StreamParams &, int64_t, \

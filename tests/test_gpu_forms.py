@@ -80,6 +80,28 @@ def test_short_frames_leave_the_wide_form_by_blocks_per_sm(K, f, v, per_sm, few)
     assert (s.form == vd.VD_FORM_FEW_FRAMES) == few, s.form
 
 
+@pytest.mark.parametrize("radix", [2, 4])
+@pytest.mark.parametrize("K,lanes,pairs_per_block", [(7, 1, 128), (9, 4, 32)])
+def test_one_wave_keeps_three_blocks_per_sm_beyond_the_deep_ring(K, lanes, pairs_per_block, radix):
+    """As many blocks as the deep traceback ring leaves resident (two per SM for
+    these shapes, three for K=7 radix 4), and one more, which has to take the form of three."""
+    t = vd.VdTune()
+    t.lanes, t.form = lanes, vd.VD_FORM_ONE_WAVE
+    code, f, v = vd.Code(K, GENS[K]), 32, 8
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+
+    def blocks_per_sm(blocks):
+        n = blocks * pairs_per_block * 2 * f
+        return n, vd.vd_decode_shape(code.handle, vd.VD_LLR_S8, n, f, v, radix, 0, t).blocks_per_sm
+
+    deep = 3 if (K, radix) == (7, 4) else 2
+    assert blocks_per_sm(deep * sm)[1] == deep
+    n, after = blocks_per_sm(deep * sm + 1)
+    assert after == 3
+    s = compare(K, n - 45, f, v, True, False, seed=n, radix=radix, tune=t)
+    assert s.blocks == deep * sm + 1
+
+
 @pytest.mark.parametrize("form", [vd.VD_FORM_PERSISTENT, vd.VD_FORM_ONE_WAVE])
 @pytest.mark.parametrize("K,lanes", [(7, 1), (7, 2), (7, 4), (9, 4), (9, 8)])
 def test_radix_4_in_both_named_forms(K, lanes, form):
