@@ -1,26 +1,22 @@
 // fp16-LLR / fp32-metric stream kernel instantiations: a frame pair over 4
 // lanes (K=7), 16 or 8 (K=9).  The caller's names of these forms
 // (vd_tune.lanes) are 2 and 8.
-#include "vd_launch.h"
+#include "vd_variants.cuh"
 #include "vd_stream_f32.cuh"
 
 namespace vd {
 
 namespace {
 
-template <int K> struct F32Of;
-template <> struct F32Of<7> { static constexpr int BETA = 2; static constexpr uint64_t GENS = GENS_K7; };
-template <> struct F32Of<9> { static constexpr int BETA = 3; static constexpr uint64_t GENS = GENS_K9; };
-
 template <int K, int L>
 cudaError_t launch(const StreamParams &p, int64_t blocks, cudaStream_t st) {
-    stream_kernel_f32<K, F32Of<K>::BETA, F32Of<K>::GENS, L, kThreads><<<(unsigned)blocks, kThreads, 0, st>>>(p);
+    stream_kernel_f32<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L, kThreads><<<(unsigned)blocks, kThreads, 0, st>>>(p);
     return cudaGetLastError();
 }
 
 template <int K, int L>
 F32Geom geom() {
-    using Cfg = StreamCfgF32<K, F32Of<K>::BETA, F32Of<K>::GENS, L>;
+    using Cfg = StreamCfgF32<K, CodeOf<K>::BETA, CodeOf<K>::GENS, L>;
     F32Geom g;
     g.geom.U = Cfg::U;
     g.geom.NW = Cfg::NW;

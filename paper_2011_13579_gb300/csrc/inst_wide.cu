@@ -1,20 +1,19 @@
 // Wide kernel instantiations (vd_wide.cuh): K=7 with 8 lanes per frame pair, K=9 with 32.
 #include <atomic>
 
-#include "vd_launch.h"
+#include "vd_variants.cuh"
 #include "vd_wide.cuh"
 
 namespace vd {
 
 namespace {
 
-template <int K> struct WideOf;
-template <> struct WideOf<7> { static constexpr int BETA = 2, L = 8; static constexpr uint64_t GENS = GENS_K7; };
-template <> struct WideOf<9> { static constexpr int BETA = 3, L = 32; static constexpr uint64_t GENS = GENS_K9; };
+template <int K> constexpr int kLanes = K == 7 ? 8 : 32;
+template <int K> using CfgOf = WideCfg<K, CodeOf<K>::BETA, CodeOf<K>::GENS, kLanes<K>>;
 
 template <int K>
 bool plan(const WideParams &in, WideParams *out, int64_t *blocks, size_t *smem, bool *full) {
-    using Cfg = WideCfg<K, WideOf<K>::BETA, WideOf<K>::GENS, WideOf<K>::L>;
+    using Cfg = CfgOf<K>;
     WideParams p = in;
     const int64_t span = p.f + 2 * p.v, wmax = p.T < span ? p.T : span;
     if (wmax > (1 << 20)) return false;
@@ -23,7 +22,7 @@ bool plan(const WideParams &in, WideParams *out, int64_t *blocks, size_t *smem, 
     p.rec0 = (int32_t)((p.wpad - kept) / Cfg::U * (Cfg::U / Cfg::ES));
     const size_t pair = Cfg::pair_bytes(p.wpad, p.rec0);
     if (pair > kWideSmemMax) return false;
-    constexpr int G = 32 / WideOf<K>::L;
+    constexpr int G = 32 / kLanes<K>;
     const int ppw = pair * G <= kWideSmemMax ? G : 1;   // frames too long for that: one pair per warp
     *blocks = (p.n_pairs + ppw - 1) / ppw;
     *smem = pair * (size_t)ppw;
@@ -32,24 +31,11 @@ bool plan(const WideParams &in, WideParams *out, int64_t *blocks, size_t *smem, 
     return true;
 }
 
-// More than 48 KB of shared memory needs the kernel's opt-in, once per device.
-template <typename Kern>
-cudaError_t opt_in(Kern kern, std::atomic<uint64_t> &done) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const uint64_t bit = dev < 64 ? (1ull << dev) : 0ull;
-    if (bit && (done.load(std::memory_order_acquire) & bit)) return cudaSuccess;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmemMax);
-    if (e == cudaSuccess && bit) done.fetch_or(bit, std::memory_order_acq_rel);
-    return e;
-}
-
 template <int K, int PPW>
 cudaError_t launch(const WideParams &p, int64_t blocks, size_t smem, cudaStream_t st) {
-    auto kern = wide_kernel<K, WideOf<K>::BETA, WideOf<K>::GENS, WideOf<K>::L, PPW>;
+    auto kern = wide_kernel<K, CodeOf<K>::BETA, CodeOf<K>::GENS, kLanes<K>, PPW>;
     static std::atomic<uint64_t> done{0};
-    const cudaError_t e = opt_in(kern, done);
+    const cudaError_t e = opt_in_smem(kern, kWideSmemMax, done);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)blocks, 32, smem, st>>>(p);
     return cudaGetLastError();
@@ -59,8 +45,7 @@ constexpr int kSplitWarps = 4;
 
 template <int K>
 bool split(const WideParams &in, int n_sm, SplitParams *out, int *ranks, size_t *smem) {
-    using W_ = WideOf<K>;
-    using Cfg = WideCfg<K, W_::BETA, W_::GENS, W_::L>;
+    using Cfg = CfgOf<K>;
     const int64_t span = in.f + 2 * in.v, wmax = in.T < span ? in.T : span;
     if (wmax > (1 << 20)) return false;
     const int nc = (int)((wmax + Cfg::U - 1) / Cfg::U);
@@ -72,9 +57,9 @@ bool split(const WideParams &in, int n_sm, SplitParams *out, int *ranks, size_t 
     bool have = false;
     for (int r = 1; r <= 8; r *= 2) {
         if (in.n_win * r > per_sm * n_sm) break;
-        const int nseg = r * kSplitWarps * 2 * (32 / W_::L);
+        const int nseg = r * kSplitWarps * 2 * (32 / kLanes<K>);
         const int S = (nc + nseg - 1) / nseg;
-        const size_t bytes = (size_t)SplitSmem<K, W_::BETA, W_::GENS, W_::L>(kSplitWarps, S, kSplitWarmup).total * 4u;
+        const size_t bytes = (size_t)SplitSmem<K, CodeOf<K>::BETA, CodeOf<K>::GENS, kLanes<K>>(kSplitWarps, S, kSplitWarmup).total * 4u;
         if (bytes > kWideSmemMax) continue;
         have = true;
         out->S = S;
@@ -99,9 +84,9 @@ bool split(const WideParams &in, int n_sm, SplitParams *out, int *ranks, size_t 
 
 template <int K>
 cudaError_t launch_s(const SplitParams &p, int ranks, size_t smem, cudaStream_t st) {
-    auto kern = split_kernel<K, WideOf<K>::BETA, WideOf<K>::GENS, WideOf<K>::L, 32 * kSplitWarps>;
+    auto kern = split_kernel<K, CodeOf<K>::BETA, CodeOf<K>::GENS, kLanes<K>, 32 * kSplitWarps>;
     static std::atomic<uint64_t> done{0};
-    const cudaError_t e = opt_in(kern, done);
+    const cudaError_t e = opt_in_smem(kern, kWideSmemMax, done);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.n_win * ranks));
@@ -119,7 +104,7 @@ cudaError_t launch_s(const SplitParams &p, int ranks, size_t smem, cudaStream_t 
 
 }  // namespace
 
-int wide_lanes(int K) { return K == 7 ? WideOf<7>::L : WideOf<9>::L; }
+int wide_lanes(int K) { return K == 7 ? kLanes<7> : kLanes<9>; }
 
 bool split_plan(int K, const WideParams &in, int n_sm, SplitParams *out, int *ranks, size_t *smem) {
     return K == 7 ? split<7>(in, n_sm, out, ranks, smem) : K == 9 ? split<9>(in, n_sm, out, ranks, smem) : false;

@@ -634,7 +634,6 @@ extern "C" vd_status vd_decode(const vd_code *c, const void *d_llr, int llr_type
 
     vd::StreamParams p;
     p.llr = llr;
-    p.llr_bytes = pl.T * c->beta;
     p.n_info = n_info;
     p.T = pl.T;
     p.f = f;
@@ -654,7 +653,6 @@ extern "C" vd_status vd_decode(const vd_code *c, const void *d_llr, int llr_type
     p.n_tasks = pl.n_tasks;
     if (pl.blocks > 0x7FFFFFFF) return fail(VD_EINVAL, "stream too long for one launch");
     cudaError_t e;
-    p.llr_bytes = pl.T * c->beta * (f32 ? 2 : 1);
     if (pl.form == Form::PERSISTENT) {
         void *ctr = nullptr;
         st = get_scratch(3, 256, cs, &ctr);

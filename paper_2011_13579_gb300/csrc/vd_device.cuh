@@ -49,11 +49,6 @@ __device__ __forceinline__ uint32_t min_u16x2(uint32_t a, uint32_t b) {
     asm("min.u16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
     return d;
 }
-__device__ __forceinline__ uint32_t max_s16x2(uint32_t a, uint32_t b) {
-    uint32_t d;
-    asm("max.s16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-    return d;
-}
 // max(a + b, c) per unsigned half
 __device__ __forceinline__ uint32_t addmax_u16x2(uint32_t a, uint32_t b, uint32_t c) {
     return max_u16x2(add_u16x2(a, b), c);
@@ -146,15 +141,6 @@ struct Code {
         return k == 0 ? (x & MASK) : (((x >> k) | (x << (NB - k))) & MASK);
     }
 };
-
-// Runtime alpha of a butterfly index (linear over GF(2)), for lane offsets.
-template <int K, int BETA, uint64_t GENS>
-__device__ __forceinline__ uint32_t alpha_rt(uint32_t g) {
-    uint32_t r = 2u * g, a = 0;
-#pragma unroll
-    for (int b = 0; b < BETA; ++b) a |= (uint32_t)(__popc(gen_of(GENS, b) & r) & 1) << b;
-    return a;
-}
 
 // ------------------------------------------------------------- frame plan
 

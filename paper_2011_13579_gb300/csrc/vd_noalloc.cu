@@ -158,7 +158,6 @@ extern "C" vd_status vd_decode_noalloc(const vd_code *c, const void *d_llr, int6
 
     vd::StreamParams p;
     p.llr = (const int8_t *)d_llr;
-    p.llr_bytes = T * c->beta;
     p.n_info = n_info;
     p.T = T;
     p.f = f;

@@ -51,7 +51,6 @@ namespace vd {
 
 struct StreamParams {
     const int8_t *llr;      // depunctured received LLRs, [T][beta], int8
-    int64_t llr_bytes;      // T * beta
     int64_t n_info, T, f, v;
     int64_t n_win, n_pairs;
     uint32_t flags;         // bit0: terminated, bit1: start state unknown
@@ -270,15 +269,16 @@ __device__ __forceinline__ uint32_t min_tree(const uint32_t (&v)[N]) {
 // Backward procedure (Algorithm 2) for one pair of frames, resumable: it walks
 // groups of K-1 stages (so the phase of every stage in a group is a
 // compile-time constant) from Wpad-1 down to the frames' first decoded
-// stages.  A persistent warp calls step() once per chunk of the NEXT frame
+// stages.  A persistent warp calls step() after every second chunk of the NEXT frame
 // pair's forward pass, so the traceback's dependent chain and its memory
-// latency hide behind forward work.  The survivor words of the next two
-// groups are copied into a per-warp shared-memory staging area by cp.async
+// latency hide behind forward work.  The survivor records of the groups walked next (two, or
+// 2 D: see D below) are copied into a per-warp shared-memory staging area by cp.async
 // while earlier groups are walked; the per-lane state lives in shared memory
-// between steps.  Every lane of a group follows both frames; the lane that
-// owns the current register supplies its decision bit (one shuffle).
-// Survivor words: bit (r & 31) of word (r >> 5) holds register r of the lane
-// (r & 15 at bit 16h when a lane has 16 registers or fewer), frame 0 first.
+// between steps.  One lane per pair follows both frames.  With several lanes and embedded
+// decisions, lanes 0 and 1 of a group (and those that repeat them) follow one frame each and read
+// any lane's records from the staging.  In the fp32 form (a decision word per stage and
+// frame: bit (r & 31) of word (r >> 5) for register r, or bit r and 16 + r of one word for lanes of 16 registers)
+// every lane follows both frames and the lane that owns the current register supplies its bit by a shuffle.
 
 // All fields are 32-bit words (pointers and the 64-bit bit accumulator are
 // split in two): 23 words, an odd stride, so the per-thread records in shared

@@ -7,7 +7,7 @@
 // Decisions: d = (c_odd >= c_even), read from the sign of c_odd - c_even
 // computed from the same rounded candidates the maximum uses (an exact tie
 // gives +0, so the odd predecessor wins it, as in Algorithm 1).  The metric of
-// state 0 is subtracted from every metric every normalisation period, which
+// state 0 is subtracted from every metric every chunk, which
 // keeps magnitudes (and so rounding) small; the reset start gives every state
 // but 0 the metric -1e30, which no finite path metric approaches.
 #pragma once
@@ -27,7 +27,6 @@ struct StreamCfgF32 {
     static constexpr int U = chunk_stages(K, 2 * BETA);   // 2 bytes per LLR
     static constexpr int UW = U * BETA / 2;               // 32-bit words per chunk per frame
     static constexpr int NW = NR / 16;                    // survivor words per lane per stage
-    static constexpr int NORM_CHUNKS = 1;
     static_assert(NR == 16 || NR == 32, "half a decision word or a word per frame and lane");
     static_assert(C::lv() == (1u << BETA) - 1u && C::mv() == (1u << BETA) - 1u, "complement branch outputs");
     // output b at phase ph: the lane bits whose parity flips it
