@@ -121,7 +121,9 @@ int vd_code_supported(int K, int beta, const uint32_t *gens_octal);
  * of Sec. III.  Unless tune asks for lanes or a form, the kernel goes by the
  * stream: few long frames are decoded in overlapping segments at once, which
  * run again until their metrics agree with those of the frame decoded in
- * one piece; few frames spread each frame pair over a quarter warp (K=7) or a
+ * one piece (up to 136,704 stages for K=7 and 49,152 for K=9, what a cluster's shared memory
+ * holds: a longer frame is one serial chain of its stages, hundreds of times slower); few
+ * frames spread each frame pair over a quarter warp (K=7) or a
  * warp (K=9); both keep their survivors in shared memory.  Longer streams take a
  * kernel with one lane group per frame pair, or a persistent one whose warps
  * pull tasks and trace one task back while decoding the next forward.  All

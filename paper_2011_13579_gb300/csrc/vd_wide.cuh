@@ -529,7 +529,8 @@ __global__ void __launch_bounds__(32, 8) wide_kernel(const WideParams p) {
 // What bounds it: the warm-up and the segment, (16 + S) (K-1) stages of 80
 // (K=7) or 100 (K=9) cycles, and some five barriers of the cluster.  Four warps a block, one
 // per scheduler (a second one on a scheduler costs 28 cycles a stage); clusters of 1 to 8
-// blocks, as wide as keeps S at half the warm-up.  Measured (us per vd_decode
+// blocks, as wide as keeps S at half the warm-up.  A frame of more than 8 (K=7: 256, K=9: 64 segments)
+// times the chunks that fit a block, 136,704 or 49,152 stages, is left to the other forms.  Measured (us per vd_decode
 // call, this form / wide / one lane per pair): K=7 full length, terminated, 3 dB, 4,096
 // bits 14.7 / 209 / 1172, 30,000 bits 18.7 / - / 8452; K=9, 4,096 bits 20.8 / - /
 // 2148; at 0 dB, where some segments run twice, 28.9 and 33.0.
