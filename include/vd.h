@@ -202,7 +202,8 @@ typedef struct vd_shape {
 } vd_shape;
 
 /*
- * What vd_decode runs for these arguments on the current device.  No launch, no
+ * What vd_decode runs for these arguments on the current device (a stream that is being
+ * captured, or for which no scratch can be allocated, may take VD_FORM_FEW_FRAMES instead, which needs none).  No launch, no
  * allocation.  n_info > 0; other errors as vd_decode.
  */
 vd_status vd_decode_shape(const vd_code *code, int llr_type, int64_t n_info, int f, int v, int radix, uint32_t flags,

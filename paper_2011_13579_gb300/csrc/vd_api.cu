@@ -318,6 +318,8 @@ struct Plan {
     vd::WideParams wide;       // WIDE (without pointers)
     int ranks;                 // SPLIT: blocks per frame
     bool wide_full;            // WIDE: a whole warp's pairs per block
+    bool wide_fits;            // WIDE can take the stream, though another form may be faster
+    int64_t wide_blocks;
     size_t smem;               // SPLIT, WIDE
 };
 
@@ -380,12 +382,12 @@ constexpr double kWideWavesK7 = 3.5, kWideWavesK9 = 2.6;
 // v = 42: 21 80.4 / 88.6, 26 92.8 / 88.8.
 constexpr int64_t kWideBlocksK7 = 38, kWideBlocksK9 = 24;
 
-bool take_wide(int K, int64_t blocks, size_t smem) {
-    const int64_t n_sm = sm_count();
+// Past that the form still stands in where no scratch can be had: it needs none.
+bool wide_within_waves(int K, int64_t blocks, size_t smem) {
     const int64_t per_sm = (int64_t)((228u * 1024u) / (smem + 1024u));   // 228 KB an SM, 1 KB of it reserved per block
-    return (double)blocks <= (K == 7 ? kWideWavesK7 : kWideWavesK9) * (double)(n_sm * std::max<int64_t>(1, per_sm)) &&
-           blocks <= (K == 7 ? kWideBlocksK7 : kWideBlocksK9) * n_sm;
+    return (double)blocks <= (K == 7 ? kWideWavesK7 : kWideWavesK9) * (double)(sm_count() * std::max<int64_t>(1, per_sm));
 }
+bool wide_is_faster(int K, int64_t blocks) { return blocks <= (K == 7 ? kWideBlocksK7 : kWideBlocksK9) * sm_count(); }
 
 size_t wave_scratch(int64_t n_pairs, int lanes, int64_t wmax, const vd::KernelGeom &g, int64_t *blocks) {
     *blocks = (n_pairs * lanes + vd::kThreads - 1) / vd::kThreads;
@@ -455,6 +457,7 @@ vd_status make_plan(const vd_code *c, int64_t n_info, int f, int v, int radix, u
     if (wmax > (1 << 30)) return fail(VD_EINVAL, "frame too long (%lld stages)", (long long)wmax);
     pl->form = Form::WAVE;
     pl->surv_bytes = 0;
+    pl->wide_fits = false;
     const int form = tune ? tune->form : 0;
     if (f32) {
         const vd::F32Geom g = vd::geom_f32(c->K, pl->n_pairs, sm_count());
@@ -474,9 +477,11 @@ vd_status make_plan(const vd_code *c, int64_t n_info, int f, int v, int radix, u
             pl->form = Form::SPLIT;
             return VD_OK;
         }
-        if (vd::wide_plan(c->K, wp, &pl->wide, &pl->blocks, &pl->smem, &pl->wide_full) &&
-            take_wide(c->K, pl->blocks, pl->smem)) {
+        pl->wide_fits = vd::wide_plan(c->K, wp, &pl->wide, &pl->wide_blocks, &pl->smem, &pl->wide_full) &&
+                        wide_within_waves(c->K, pl->wide_blocks, pl->smem);
+        if (pl->wide_fits && wide_is_faster(c->K, pl->wide_blocks)) {
             pl->form = Form::WIDE;
+            pl->blocks = pl->wide_blocks;
             return VD_OK;
         }
         // K=7 radix 4 takes radix-2 steps here (the same bits): us, radix-4 / radix-2
@@ -611,26 +616,33 @@ extern "C" vd_status vd_decode(const vd_code *c, const void *d_llr, int llr_type
         llr = (const int8_t *)buf;
     }
 
-    if (pl.form == Form::SPLIT || pl.form == Form::WIDE) {
-        if (pl.form == Form::SPLIT) {
-            pl.split.llr = llr;
-            pl.split.out = d_out;
-            pl.split.pm_out = d_pm;
-        } else {
-            pl.wide.llr = llr;
-            pl.wide.out = d_out;
-            pl.wide.pm_out = d_pm;
-        }
-        const cudaError_t e = pl.form == Form::SPLIT
-                                  ? vd::launch_split(c->K, pl.split, pl.ranks, pl.smem, cs)
-                                  : vd::launch_wide(c->K, pl.wide, pl.blocks, pl.smem, pl.wide_full, cs);
-        if (e != cudaSuccess) return cuda_fail(e, "decode launch");
-        return VD_OK;
+    if (pl.form == Form::SPLIT) {
+        pl.split.llr = llr;
+        pl.split.out = d_out;
+        pl.split.pm_out = d_pm;
+        const cudaError_t e = vd::launch_split(c->K, pl.split, pl.ranks, pl.smem, cs);
+        return e == cudaSuccess ? VD_OK : cuda_fail(e, "decode launch");
     }
-
+    // The wide form needs no allocation: it also takes the streams it can where
+    // none may be made (capture) or none can (the pool cannot grow).
     void *surv = nullptr;
-    st = get_scratch(0, pl.surv_bytes, cs, &surv);
-    if (st != VD_OK) return st;
+    if (pl.form != Form::WIDE && pl.wide_fits) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(cs, &cap) != cudaSuccess) cudaGetLastError();
+        if (cap != cudaStreamCaptureStatusNone) pl.form = Form::WIDE;
+    }
+    if (pl.form != Form::WIDE) {
+        st = get_scratch(0, pl.surv_bytes, cs, &surv);
+        if (st == VD_ENOMEM && pl.wide_fits) pl.form = Form::WIDE;
+        else if (st != VD_OK) return st;
+    }
+    if (pl.form == Form::WIDE) {
+        pl.wide.llr = llr;
+        pl.wide.out = d_out;
+        pl.wide.pm_out = d_pm;
+        const cudaError_t e = vd::launch_wide(c->K, pl.wide, pl.wide_blocks, pl.smem, pl.wide_full, cs);
+        return e == cudaSuccess ? VD_OK : cuda_fail(e, "decode launch");
+    }
 
     vd::StreamParams p;
     p.llr = llr;

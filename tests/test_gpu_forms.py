@@ -80,6 +80,27 @@ def test_short_frames_leave_the_wide_form_by_blocks_per_sm(K, f, v, per_sm, few)
     assert (s.form == vd.VD_FORM_FEW_FRAMES) == few, s.form
 
 
+@pytest.mark.parametrize("K,n", [(7, 3_000_000), (9, 600_000)])
+def test_short_frames_can_be_captured_without_scratch(K, n):
+    """A first call for short frames inside a stream capture, where nothing may be allocated."""
+    f, v = 32, 6
+    code = vd.Code(K, GENS[K])
+    q = synth.make_stream(np.random.Generator(np.random.PCG64(n)), K, GENS[K], n, 2.0, False).s8()
+    llr = torch.from_numpy(q.view(np.uint8)).cuda()
+    want = vd.decode(code, llr, n, f, v)
+    vd.vd_sync()
+    assert vd.vd_decode_shape(code.handle, vd.VD_LLR_S8, n, f, v).form != vd.VD_FORM_FEW_FRAMES
+    out = torch.full_like(want, -1)
+    torch.cuda.synchronize()
+    vd.vd_release_scratch()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        vd.decode(code, llr, n, f, v, out=out)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+
+
 @pytest.mark.parametrize("radix", [2, 4])
 @pytest.mark.parametrize("K,lanes,pairs_per_block", [(7, 1, 128), (9, 4, 32)])
 def test_one_wave_keeps_three_blocks_per_sm_beyond_the_deep_ring(K, lanes, pairs_per_block, radix):
